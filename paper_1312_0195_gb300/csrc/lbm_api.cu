@@ -129,7 +129,14 @@ struct lbm_grid {
     double *h_result = nullptr;      // pinned [4]
     GridLaunch L{};
     int64_t t = 0;
-    std::map<std::tuple<int, int, int>, std::pair<cudaGraphExec_t, int>> graphs;
+    int sms = 1;
+    bool fused = false;              // several steps per pass (multistep.cu) where a call takes several
+    struct Graph {
+        cudaGraphExec_t exec;
+        int kernels;                 // launches it holds
+        int cur;                     // buffer that holds the state after it
+    };
+    std::map<std::tuple<int, int, int, int>, Graph> graphs;
 };
 
 namespace lbm {
@@ -204,25 +211,46 @@ static cudaError_t enqueue_moments(const lbm_grid *g, int cur_idx, int prev_idx,
     }
 }
 
-// Graph of n fused steps starting from buf[parity], optionally followed by the
-// residual pass (moments of the last two states, reduction, copy to pinned host).
-static lbm_status get_graph(lbm_grid *g, int n, int parity, int check, cudaGraphExec_t *out, int *nk)
+// nlev steps in one pass over memory (multistep.cu).
+static cudaError_t enqueue_multi(const lbm_grid *g, int src_idx, int nlev, cudaStream_t st)
 {
-    auto key = std::make_tuple(n, parity, check);
+    const void *src = g->buf[src_idx];
+    void *dst = g->buf[1 - src_idx];
+    const bool walls = g->p.bc == LBM_BC_WALLS_Y;
+    if (g->p.storage == LBM_F16) {
+        auto a = make_args<__half, float>(g, src, dst);
+        return launch_multistep(LBM_F16, g->coef_mode, g->has_g, walls, &a, nlev, g->sms, st);
+    }
+    auto a = make_args<float, float>(g, src, dst);
+    return launch_multistep(LBM_F32, g->coef_mode, g->has_g, walls, &a, nlev, g->sms, st);
+}
+
+// Graph of n steps starting from buf[parity], optionally followed by the residual pass (moments of
+// the last two states, reduction, copy to pinned host). Where the grid fuses steps, the passes take
+// MULTISTEP_MAX steps each; with `pair` the last step is one of its own, so that the two
+// buffers end up holding the last two states (the residual and a checkpoint read both).
+static lbm_status get_graph(lbm_grid *g, int n, int parity, int check, int pair, lbm_grid::Graph *out)
+{
+    if (!g->fused) pair = 0;
+    auto key = std::make_tuple(n, parity, check, pair);
     auto it = g->graphs.find(key);
     if (it != g->graphs.end()) {
-        *out = it->second.first;
-        *nk = it->second.second;
+        *out = it->second;
         return LBM_OK;
     }
     cudaGraph_t graph = nullptr;
     LBM_CUDA(cudaStreamBeginCapture(g->cap, cudaStreamCaptureModeThreadLocal));
     cudaError_t err = cudaSuccess;
     int idx = parity, kernels = 0;
-    for (int i = 0; i < n && err == cudaSuccess; ++i) {
-        err = enqueue_step(g, idx, g->cap);
+    for (int left = n; left > 0 && err == cudaSuccess; ++kernels) {
+        int take = 1;
+        if (g->fused) {
+            take = left - (pair || check ? 1 : 0);
+            take = take < 1 ? 1 : (take > MULTISTEP_MAX ? MULTISTEP_MAX : take);
+        }
+        err = take > 1 ? enqueue_multi(g, idx, take, g->cap) : enqueue_step(g, idx, g->cap);
         idx = 1 - idx;
-        ++kernels;
+        left -= take;
     }
     if (check && err == cudaSuccess) {
         err = enqueue_moments(g, idx, 1 - idx, nullptr, nullptr, nullptr, g->cap);
@@ -245,9 +273,7 @@ static lbm_status get_graph(lbm_grid *g, int n, int parity, int check, cudaGraph
         cudaGetLastError();
         return fail(LBM_ECUDA, "graph instantiation failed: %s", cudaGetErrorString(e3));
     }
-    g->graphs[key] = {exec, kernels};
-    *out = exec;
-    *nk = kernels;
+    *out = g->graphs[key] = {exec, kernels, idx};
     return LBM_OK;
 }
 
@@ -356,7 +382,7 @@ static lbm_status autotune(lbm_grid *g)
 static void free_grid(lbm_grid *g)
 {
     if (!g) return;
-    for (auto &kv : g->graphs) cudaGraphExecDestroy(kv.second.first);
+    for (auto &kv : g->graphs) cudaGraphExecDestroy(kv.second.exec);
     g->graphs.clear();
     cudaFree(g->buf[0]);
     cudaFree(g->buf[1]);
@@ -415,6 +441,8 @@ lbm_status grid_create_impl(const lbm_params *p, const float *kappa_dev, const d
 
     // launch shapes: persistent step grid, fixed moment grid (fixed reduction order)
     const int sms = sm_count(g->dev);
+    g->sms = sms;
+    g->fused = !std::getenv("LBM_STEP_VEC") && multistep_ok(p->storage, g->coef_mode, p->nx, p->ny, p->force_model);
     const int vec = step_vec(p->storage, p->nx);
     const int64_t chunks = n / vec;
     g->L.step_threads = 256;
@@ -424,7 +452,7 @@ lbm_status grid_create_impl(const lbm_params *p, const float *kappa_dev, const d
                                                           p->bc == LBM_BC_WALLS_Y, p->nx, g->L.step_threads);
     g->L.step_blocks = (int)(want < cap ? (want < 1 ? 1 : want) : cap);
     // LBM_STEP_VEC=v selects another built cells-per-thread variant of the step (the arithmetic per
-    // cell is the same in every variant) and turns the autotuner off for this grid
+    // cell is the same in every variant) and turns the autotuner and the fused passes off for this grid
     if (const char *ev = std::getenv("LBM_STEP_VEC")) {
         const int v = std::atoi(ev);
         if (step_vec_ok(p->storage, p->nx, v)) {
@@ -556,16 +584,15 @@ lbm_status lbm_step(lbm_grid *g, int64_t max_steps, double tol_rel, int32_t chec
                 check = 1;
             }
         }
-        cudaGraphExec_t ex = nullptr;
-        int nk = 0;
-        lbm_status s = get_graph(g, (int)n, g->cur, check, &ex, &nk);
+        lbm_grid::Graph gr{};
+        lbm_status s = get_graph(g, (int)n, g->cur, check, n == left || tol_rel > 0.0, &gr);
         if (s != LBM_OK) return s;
-        LBM_CUDA(cudaGraphLaunch(ex, g->stream));
-        count_launches(nk);
+        LBM_CUDA(cudaGraphLaunch(gr.exec, g->stream));
+        count_launches(gr.kernels);
         g->t += n;
         done += n;
         left -= n;
-        if (n & 1) g->cur = 1 - g->cur;
+        g->cur = gr.cur;
         if (check) {
             checked = true;
             if (tol_rel > 0.0) {      // the stop test needs the value now; otherwise read it at the end

@@ -75,6 +75,14 @@ int step_vec(int storage, int nx);   // cells per thread used for this storage a
 int step_blocks_per_sm(int storage, int coef_mode, bool gfield, bool walls, int nx, int threads, int vec = 0);
 bool step_vec_ok(int storage, int nx, int vec);   // is this cells-per-thread variant built and usable
 
+// ---- several steps per pass (multistep.cu) ---------------------------------------
+constexpr int MULTISTEP_MAX = 4;        // steps one pass fuses at most
+constexpr int MULTISTEP_MIN_ROWS = 4;   // rows of a warp's segment at least: fewer repeat more halo rows than
+                                        // they gain in parallel warps (256 x 256: 2.9 us a step at 4, 3.3 at 2)
+bool multistep_ok(int storage, int coef_mode, int nx, int ny, int guo);
+cudaError_t launch_multistep(int storage, int coef_mode, bool gfield, bool walls, const void *args, int nlev, int sms,
+                             cudaStream_t st);
+
 // ---- launch counter (lbm_api.cu) ----------------------------------------------
 void count_launches(int64_t n);
 

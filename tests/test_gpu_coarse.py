@@ -184,3 +184,29 @@ def test_fiveblock_brinkman_kstar_beats_kstar_err():
     e_good, e_bad = _rel(uc, uf), _rel(ue, uf)
     print(f"E6 coarse vs fine: rel L2 u with K* {e_good:.3e}, with K*err {e_bad:.3e}")
     assert e_good < e_bad
+
+
+@pytest.mark.parametrize("nx,ny", [(56, 8), (65, 31), (20, 130)])
+def test_coarse_run_fused_passes_equal_single_steps_bitwise(nx, ny, monkeypatch):
+    """The coarse run's tensor drag in passes of several steps against the one-step kernel."""
+    import torch
+    import paper_1312_0195_gb300 as lbm
+    g = torch.Generator().manual_seed(nx)
+    K = 0.05 * torch.rand((ny, nx, 4), generator=g, dtype=torch.float64)
+    K[..., 0] += 0.2
+    K[..., 3] += 0.2
+    field = torch.rand((2, ny, nx), generator=g).cuda() * 1e-6
+    for bc in (lbm.LBM_BC_PERIODIC, lbm.LBM_BC_WALLS_Y):
+        for force in (None, field):
+            got = []
+            for single in (False, True):
+                if single:
+                    monkeypatch.setenv("LBM_STEP_VEC", "1")
+                else:
+                    monkeypatch.delenv("LBM_STEP_VEC", raising=False)
+                out = [torch.empty((ny, nx), device="cuda") for _ in range(3)]
+                lbm.lbm_coarse_run(lbm.Params(nx=4 * nx, ny=4 * ny, tau=1.0, gx=1e-6, bc=bc), 4, K.cuda(), force, 777,
+                                   0.0, 64, *out)
+                got.append(out)
+            for a, b in zip(*got):
+                assert torch.equal(a, b)

@@ -373,3 +373,32 @@ def test_every_cells_per_thread_variant_agrees_bitwise(storage, vecs, monkeypatc
                 states[v] = st.cpu().numpy()
         for v in vecs[1:]:
             np.testing.assert_array_equal(states[v], states[vecs[0]])
+
+
+@pytest.mark.parametrize("storage", [0, 1])
+@pytest.mark.parametrize("nx,ny", [(56, 8), (57, 9), (113, 37), (8, 64), (2, 8), (300, 101), (1024, 520)])
+def test_fused_passes_equal_single_steps_bitwise(storage, nx, ny, monkeypatch):
+    """A grid takes several steps per pass over memory; every cell's arithmetic is that of the one-step
+    kernel (LBM_STEP_VEC selects it), so states and residuals agree bit for bit. Sizes: one strip of 56
+    columns and one column more, odd rows, lattices narrower than a strip, several row segments."""
+    import torch
+    lbm = _lbm()
+    kap = torch.from_numpy(synth.lognormal_kappa(nx, ny, 4.0, 1.5, seed=nx + ny).astype(np.float32)).cuda()
+    field = torch.rand((2, ny, nx), generator=torch.Generator().manual_seed(3)).cuda() * 1e-6
+    for walls in (False, True):
+        for force in (None, field):
+            got = []
+            for single in (False, True):
+                if single:
+                    monkeypatch.setenv("LBM_STEP_VEC", "1")
+                else:
+                    monkeypatch.delenv("LBM_STEP_VEC", raising=False)
+                p = lbm.Params(nx=nx, ny=ny, tau=0.7, gx=1e-6, gy=3e-7, storage=storage,
+                               bc=lbm.LBM_BC_WALLS_Y if walls else lbm.LBM_BC_PERIODIC)
+                with lbm.Grid(p, kap, force) as G:
+                    resid = [G.step(n, 0.0, check)[1] for n, check in ((1, 0), (2, 0), (7, 3), (64, 64), (1030, 100))]
+                    st = torch.empty(lbm.lbm_grid_state_bytes(G.handle), dtype=torch.uint8, device="cuda")
+                    lbm.lbm_grid_save_state(G.handle, st)
+                    got.append((resid, st.cpu().numpy()))
+            assert got[0][0] == got[1][0]
+            np.testing.assert_array_equal(got[0][1], got[1][1])
