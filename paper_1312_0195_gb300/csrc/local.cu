@@ -3,7 +3,8 @@
 // G1 = (G, 0) and G2 = (0, G), each until its volume-averaged velocity settles,
 // then K* from Eq. 17. All jobs of a batch run in ONE persistent launch.
 //
-// Design (one CTA per SM, 1024 threads):
+// Leaves from rest in FP32 whose side is a multiple of 4 are solved by the kernel of local_reg.cuh; this
+// file's solver takes the others, with the same results. Its design (one CTA per SM, 1024 threads):
 //  * A CTA owns CMAX = 4096 lattice cells in shared memory and works on one
 //    leaf size s at a time: it holds nslots = min(CMAX / s^2, MAXSLOTS) jobs of
 //    that size side by side ("slots"). Jobs are popped from a per-size device
@@ -93,6 +94,7 @@ struct LocalArgs {
     int *worst;               // [1] (zeroed)
     int *abort_flag;          // [1] (zeroed)
     unsigned long long time_limit_ns;
+    int skip_reg;             // 1: sides of the register solver (local_reg.cuh) are not taken here
 };
 
 struct Slot {
@@ -142,6 +144,14 @@ void cell_consts(LocalArgs &a)
 template <typename T> __device__ __forceinline__ T kc(const LocalArgs &a, int i);
 template <> __device__ __forceinline__ float kc<float>(const LocalArgs &a, int i) { return a.kf[i]; }
 template <> __device__ __forceinline__ double kc<double>(const LocalArgs &a, int i) { return a.kd[i]; }
+
+}  // namespace
+}  // namespace lbm
+
+#include "local_reg.cuh"
+
+namespace lbm {
+namespace {
 
 // Eqs. 6, 16, 2 and 13 for one cell in deviation form with the D2Q9 sums written out (a product
 // with a zero velocity component is not free in IEEE arithmetic): moments, r = j + eps rho G / 2,
@@ -681,6 +691,7 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) local_keff_kernel(LocalArgs 
 
     for (int cls = 0; cls < s_nclass; ++cls) {
         const int s = s_csize[cls], s2 = s * s;
+        if (a.skip_reg && reg_side(s)) continue;
         int nslots = CMAX / s2;
         if (nslots > MAXSLOTS) nslots = MAXSLOTS;
         const int ncell = nslots * s2;
@@ -1049,6 +1060,35 @@ __global__ void lg_finish_kernel(int64_t n, const int *pos, const float *kuni, c
     for (int q = 0; q < 4; ++q) keff[4 * i + q] = k[q];
 }
 
+// Launches the solvers of a batch on `blocks` CTAs: from rest in FP32, sides that are multiples of 4
+// go to the register solver (1.2 to 2.3 times the rate of the shared-memory one at every such side, see
+// local_reg.cuh) and the rest to the shared-memory one; everything else to the latter.
+// reg, other: whether the batch has sides of either kind (both, if only the device knows).
+cudaError_t launch_solvers(LocalArgs &a, bool f64, double tau, bool lg, int blocks, bool reg, bool other,
+                           cudaStream_t st)
+{
+    const bool use_reg = !f64 && !lg && !a.warm;
+    if (use_reg && reg) {
+        const auto kern = tau == 1.0 ? local_reg_kernel<true> : local_reg_kernel<false>;
+        const cudaError_t e =
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RegShared));
+        if (e != cudaSuccess) return e;
+        kern<<<blocks, RG_THREADS, sizeof(RegShared), st>>>(a);
+        count_launches(1);
+    }
+    if (!use_reg || other) {
+        a.skip_reg = use_reg ? 1 : 0;
+        const LocalKernel kern = lg ? local_kernel_lg(f64, tau) : local_kernel(f64, tau, a.warm);
+        const size_t smem = lg ? (f64 ? lg_smem<double>() : lg_smem<float>())
+                               : f64 ? LocalCfg<double>::SMEM : LocalCfg<float>::SMEM;
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        kern<<<blocks, LOCAL_THREADS, smem, st>>>(a);
+        count_launches(1);
+    }
+    return cudaGetLastError();
+}
+
 // what the local-global variant of the solver needs beyond the plain local problems
 struct LgInput {
     const float *state;   // coarse (drho, u, v) [2][3][nyc][nxc]
@@ -1197,26 +1237,22 @@ lbm_status local_keff_core(const lbm_params *p, const float *kappa_dev, const lb
     a.abort_flag = d_flags + 1;
 
     const bool f64 = p->storage == LBM_F64;
-    const LocalKernel kern = lg ? local_kernel_lg(f64, p->tau) : local_kernel(f64, p->tau, p->warm_start);
-    const size_t smem = lg ? (f64 ? lg_smem<double>() : lg_smem<float>())
-                           : f64 ? LocalCfg<double>::SMEM : LocalCfg<float>::SMEM;
-    LOC_CUDA2(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int dev = 0;
     LOC_CUDA2(cudaGetDevice(&dev));
     if (persistent) {
         a.nclass = (int)sizes.size();
+        bool reg = false, other = false;
         for (int c = 0; c < a.nclass; ++c) {
             a.class_off[c] = off[c];
             a.class_size[c] = sizes[c];
+            (reg_side(sizes[c]) ? reg : other) = true;
         }
         a.class_off[a.nclass] = off[a.nclass];
         a.heads = d_heads;
         int blocks = sm_count(dev);
         const int64_t max_useful = (int64_t)jobs.size();
         if (blocks > max_useful) blocks = (int)max_useful;
-        kern<<<blocks, LOCAL_THREADS, smem, st>>>(a);
-        LOC_CUDA2(cudaGetLastError());
-        count_launches(1);
+        LOC_CUDA2(launch_solvers(a, f64, p->tau, lg != nullptr, blocks, reg, other, st));
     } else {
         a.nclass = 1;
         for (int i = 0; i < n_leaves; ++i) {
@@ -1224,10 +1260,9 @@ lbm_status local_keff_core(const lbm_params *p, const float *kappa_dev, const lb
             a.class_off[1] = 2 * i + 2;
             a.class_size[0] = lv[i].size + 2 * m;
             a.heads = d_heads + i;
-            kern<<<1, LOCAL_THREADS, smem, st>>>(a);
-            LOC_CUDA2(cudaGetLastError());
+            const bool reg = reg_side(a.class_size[0]);
+            LOC_CUDA2(launch_solvers(a, f64, p->tau, lg != nullptr, 1, reg, !reg, st));
         }
-        count_launches(n_leaves);
     }
     int flags[2] = {0, 0};
     LOC_CUDA2(cudaMemcpyAsync(flags, d_flags, sizeof flags, cudaMemcpyDeviceToHost, st));
@@ -1397,21 +1432,15 @@ lbm_status launch_local_from_table(const lbm_params *p, const float *kappa_dev, 
     a.worst = table + DT_WORST;
     a.abort_flag = table + DT_ABORT;
     a.time_limit_ns = (unsigned long long)(time_limit_s * 1e9);
-    const bool f64 = p->storage == LBM_F64;
-    const LocalKernel kern = local_kernel(f64, p->tau, p->warm_start);
-    const size_t smem = f64 ? LocalCfg<double>::SMEM : LocalCfg<float>::SMEM;
+    // one CTA per SM; CTAs of an empty table find no class and return at once
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess)
+        e = launch_solvers(a, p->storage == LBM_F64, p->tau, false, sm_count(dev), true, true, st);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        return fail(LBM_ECUDA, "local solver set-up: %s", cudaGetErrorString(e));
+        return fail(LBM_ECUDA, "local solver launch: %s", cudaGetErrorString(e));
     }
-    // one CTA per SM; CTAs of an empty table find no class and return at once
-    kern<<<sm_count(dev), LOCAL_THREADS, smem, st>>>(a);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return fail(LBM_ECUDA, "local solver launch: %s", cudaGetErrorString(e));
-    count_launches(1);
     return LBM_OK;
 }
 
@@ -1647,14 +1676,11 @@ extern "C" lbm_status lbm_local_keff_batch_noalloc(const lbm_params *p, const fl
     a.worst = scr + NA_FLAGS + 1;
     a.abort_flag = scr + NA_FLAGS + 2;
     a.time_limit_ns = (unsigned long long)(g_time_limit_s * 1e9);
-    const LocalKernel kern = local_kernel(f64, p->tau, p->warm_start);
-    const size_t smem = f64 ? LocalCfg<double>::SMEM : LocalCfg<float>::SMEM;
-    NA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    bool reg = false, other = false;
+    for (int c = 0; c < a.nclass; ++c) (reg_side(a.class_size[c]) ? reg : other) = true;
     int blocks = sm_count(dev);
     if (blocks > 2 * n_leaves) blocks = 2 * n_leaves;
-    kern<<<blocks, LOCAL_THREADS, smem, st>>>(a);
-    NA_CUDA(cudaGetLastError());
-    count_launches(1);
+    NA_CUDA(launch_solvers(a, f64, p->tau, false, blocks, reg, other, st));
     int flags[2] = {0, 0};
     NA_CUDA(cudaMemcpyAsync(flags, scr + NA_FLAGS + 1, sizeof flags, cudaMemcpyDeviceToHost, st));
     NA_CUDA(cudaStreamSynchronize(st));

@@ -333,3 +333,20 @@ def test_warm_start_value_is_checked():
     with pytest.raises(lbm.LbmError) as ei:
         lbm.local_keff(lbm.Params(nx=16, ny=16, tau=1.0, warm_start=2), kap, lt, 1e-6, 0.0, 10)
     assert ei.value.status == lbm.LBM_EINVAL
+
+
+@pytest.mark.parametrize("tau,steps,k", [(1.0, 300, 64), (0.8, 130, 7), (1.0, 1, 64)])
+def test_every_side_of_the_register_solver_matches_oracle(tau, steps, k):
+    """Sides that are multiples of 4 keep their distributions in registers; each packs its rows into
+    lanes and warps in another way (a part of a warp, one, two, four or sixteen warps, with idle lanes or
+    without). 1e-4 is the FP32 bar of this file. The sides in between take the other solver in the same
+    call."""
+    kap = synth.lognormal_kappa(96, 96, 6.0, 1.0, seed=77)
+    kap[5:9, 5:9] = 0.0
+    sides = list(range(4, 65, 4)) + [5, 18, 63]
+    leaves = np.array([[(7 * s) % (97 - s), (5 * s) % (97 - s), s] for s in sides + [8, 8, 8, 12, 16, 16]], dtype=np.int32)
+    ke, st, n, worst = gpu_keff(kap, leaves, tau, 0.1, 0.9, 1e-6, 0.0, steps, k=k)
+    assert worst == 0 and (n == steps).all()
+    for i in range(len(leaves)):
+        ref = oracle_keff(kap, leaves[i], tau, 0.1, 0.9, 1e-6, 0.0, steps, k=k)
+        assert_keff_close(ke[i], ref["keff"], 1e-4)
