@@ -299,6 +299,7 @@ static lbm_status autotune(lbm_grid *g)
     const char *env = std::getenv("LBM_AUTOTUNE");
     if (env && env[0] == '0') return LBM_OK;
     if (std::getenv("LBM_STEP_VEC")) return LBM_OK;      // a variant was chosen explicitly
+    if (g->p.storage == LBM_F64) return LBM_OK;          // bound by the FP64 pipe: see grid_create_impl
     const int64_t n = (int64_t)g->p.nx * g->p.ny;
     if (n < ((int64_t)1 << 20)) return LBM_OK;      // small lattices are launch-bound: keep the default
     const bool walls = g->p.bc == LBM_BC_WALLS_Y;
@@ -445,12 +446,15 @@ lbm_status grid_create_impl(const lbm_params *p, const float *kappa_dev, const d
     g->fused = !std::getenv("LBM_STEP_VEC") && multistep_ok(p->storage, g->coef_mode, p->nx, p->ny, p->force_model);
     const int vec = step_vec(p->storage, p->nx);
     const int64_t chunks = n / vec;
-    g->L.step_threads = 256;
+    const bool f64 = p->storage == LBM_F64;
+    // FP64 is bound by its arithmetic pipe: one chunk per thread in small blocks keeps every SM busy to the
+    // end (1000 x 1000: 0.108 ms a step against 0.116 with a persistent grid's uneven last round)
+    g->L.step_threads = f64 ? 128 : 256;
     g->L.step_vec = 0;
     const int64_t want = (chunks + g->L.step_threads - 1) / g->L.step_threads;
     const int64_t cap = (int64_t)sms * step_blocks_per_sm(p->storage, g->coef_mode, g->has_g,
                                                           p->bc == LBM_BC_WALLS_Y, p->nx, g->L.step_threads);
-    g->L.step_blocks = (int)(want < cap ? (want < 1 ? 1 : want) : cap);
+    g->L.step_blocks = (int)(want < 1 ? 1 : (want < cap || f64 ? want : cap));
     // LBM_STEP_VEC=v selects another built cells-per-thread variant of the step (the arithmetic per
     // cell is the same in every variant) and turns the autotuner and the fused passes off for this grid
     if (const char *ev = std::getenv("LBM_STEP_VEC")) {
