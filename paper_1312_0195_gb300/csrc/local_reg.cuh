@@ -27,19 +27,11 @@
 // thread on 8 warps gained 5 % at side 64 and lost 3 to 12 % below.
 #pragma once
 
+#include "leaf_groups.cuh"
 #include "pair_ops.cuh"
 
 namespace lbm {
 namespace {
-
-constexpr int RG_WARPS = 16;
-constexpr int RG_THREADS = RG_WARPS * 32;
-constexpr int RG_ROWS = 4;                   // rows of a thread's block
-constexpr int RG_JOBS = 16;                  // leaves of one warp at most (side 4)
-constexpr int RG_WCELLS = 256;               // cells of the velocity scratch per warp
-
-// Does this solver take leaves (grown by the margin) of side s?
-__host__ __device__ constexpr bool reg_side(int s) { return s >= 4 && s <= 64 && s % 4 == 0; }
 
 struct RegSlot {
     int job;                                 // -1: empty
@@ -58,17 +50,6 @@ struct RegShared {
     int abort[RG_WARPS];
     unsigned long long t0;
 };
-
-// Barrier of a group of `g` warps whose first is `w0`: each (size, position) has a hardware barrier of its own.
-__device__ __forceinline__ void group_sync(int g, int w0)
-{
-    if (g == 1) {
-        __syncwarp();
-    } else {
-        const int id = g == 2 ? 1 + w0 / 2 : (g == 4 ? 9 + w0 / 4 : (g == 8 ? 13 + w0 / 8 : 15));
-        asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(g * 32) : "memory");
-    }
-}
 
 // Two cells through collide_d2q9, products and sums fused as there. ne is minus the drag fraction.
 template <bool TAU1>
@@ -112,59 +93,6 @@ __device__ __forceinline__ void collide_reg(float2 (&g)[Q], float2 ne, float2 hg
         if constexpr (TAU1) g[k] = mul2(dup2(w), q[k]);
         else g[k] = fma2(dup2(-a.kf[K_OMEGA]), fma2(dup2(-w), q[k], g[k]), g[k]);
     }
-}
-
-// What a thread knows of its leaf size.
-struct RegGeo {
-    int s, group, w0;            // side; warps of the group and its first warp
-    int jobs, job;               // leaves of the group; this lane's
-    int row, col;                // first row and first column of this thread's block
-    bool cell;                   // has cells
-    int left, right;             // lanes of the neighbouring columns
-    int below, above;            // exchange offsets (warp * 6 * 32 + lane) of the neighbouring row blocks
-    int scratch;                 // velocity scratch of this lane's leaf
-};
-
-__device__ __forceinline__ RegGeo reg_geometry(int s, int warp, int lane)
-{
-    RegGeo q;
-    const int w = s / 2, per_warp = 32 / w, blocks = s / RG_ROWS;
-    q.s = s;
-    q.group = 1;
-    q.jobs = per_warp / blocks;
-    if (q.jobs < 1) {
-        q.jobs = 1;
-        while (q.group * per_warp < blocks) q.group *= 2;
-    }
-    q.w0 = warp / q.group * q.group;
-    const int c = lane % w, b = lane / w;                    // column pair, row block within the warp
-    int rb;                                                  // row block within the leaf
-    if (q.group == 1) {
-        q.job = b / blocks;
-        rb = b - q.job * blocks;
-        q.cell = q.job < q.jobs;
-        if (!q.cell) q.job = 0;
-    } else {
-        q.job = 0;
-        rb = (warp - q.w0) * per_warp + b;
-        q.cell = b < per_warp && rb < blocks;
-    }
-    q.row = rb * RG_ROWS;
-    q.col = 2 * c;
-    q.left = q.right = lane;
-    q.below = q.above = warp * 6 * 32 + lane;
-    if (q.cell) {
-        q.left = c == 0 ? lane + w - 1 : lane - 1;
-        q.right = c == w - 1 ? lane - w + 1 : lane + 1;
-        auto place = [&](int r) {
-            if (q.group == 1) return warp * 6 * 32 + (q.job * blocks + r) * w + c;
-            return (q.w0 + r / per_warp) * 6 * 32 + (r % per_warp) * w + c;
-        };
-        q.below = place(rb == 0 ? blocks - 1 : rb - 1);
-        q.above = place(rb == blocks - 1 ? 0 : rb + 1);
-    }
-    q.scratch = q.w0 * RG_WCELLS + q.job * s * s;
-    return q;
 }
 
 // One lattice step of the group's leaves. f holds the post-collision values of this thread's rows; the rows
@@ -325,7 +253,9 @@ __global__ void __launch_bounds__(RG_THREADS, 1) local_reg_kernel(LocalArgs a)
     for (int cls = 0; cls < nclass; ++cls) {
         const int s = a.table ? a.table[DT_SIZE + cls] : a.class_size[cls];
         if (!reg_side(s)) continue;
-        const RegGeo q = reg_geometry(s, warp, lane);
+        RegGeo q = reg_geometry(s, warp, lane);
+        q.below = (q.below >> 5) * (6 * 32) + (q.below & 31);    // offsets in ex
+        q.above = (q.above >> 5) * (6 * 32) + (q.above & 31);
         const bool leader = warp == q.w0;
         RegSlot *slots = sh.slots[q.w0];
         unsigned T = 0;                              // group step

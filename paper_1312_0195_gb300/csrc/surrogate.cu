@@ -442,20 +442,14 @@ __global__ void __launch_bounds__(256) patch_base_kernel(const float *x, int n, 
 // cells is k_f (p_i - p_j + G . (x_j - x_i)) with k_f the harmonic mean of the two cells, every cell
 // conserves mass, the leaf is periodic, and a unit force drives the flow along x, then along y.
 // K* along the drive is the mean face flux. The pressure system is solved by conjugate gradients
-// with the diagonal as preconditioner, in FP32 with the cross-thread sums in FP64, to a relative
-// residual of 1e-5 (K* then agrees with an FP64 direct solve to a few 1e-6). The leaf's log K is
+// with the diagonal as preconditioner, in FP32, to a relative residual of 1e-5 or less (K* then
+// agrees with an FP64 direct solve to a few 1e-6). The leaf's log K is
 // read back from the input planes (phase plane 0 sampled every 32 / s pixels for s <= 32, the four
 // phase planes for 64 cells; above 64 cells the 64 x 64 plane stands for the leaf).
-// Leaves of up to 32 cells are solved by one warp each (darcy_small_kernel), larger ones by a
-// CTA each (darcy_big_kernel); each kernel passes over the leaves of the other kind.
+// darcy_classify_kernel lists the leaves by side; 4, 8, 16, 32 and 64 are solved by darcy_group_kernel
+// (darcy_groups.cuh), the other sides by a warp each (darcy_warp_kernel).
 constexpr int DB_N = 64;
-constexpr int DB_CELLS = DB_N * DB_N;
 constexpr int DB_MAXIT = 4000;
-constexpr int DBS_WARPS = 8;                                 // warps per CTA of the small-leaf kernel
-constexpr int DBS_CELLS = IMG * IMG;                         // cells per warp (leaves up to 32)
-constexpr size_t DBS_SMEM = (size_t)DBS_WARPS * 6 * DBS_CELLS * sizeof(float);
-constexpr int DBB_THREADS = 256;
-constexpr size_t DBB_SMEM = (size_t)6 * DB_CELLS * sizeof(float);
 
 __device__ __forceinline__ int darcy_size(const float *xi)
 {
@@ -470,42 +464,29 @@ __device__ __forceinline__ float harmonic2f(double a, double b)
     return a + b > 0.0 ? (float)(2.0 * a * b / (a + b)) : 0.0f;
 }
 
-// A group of NT threads solving one leaf: one warp (NT = 32) or the whole CTA.
-template <int NT> struct DarcyGroup {
-    __device__ static int rank() { return threadIdx.x % NT; }
-    __device__ static void sync()
-    {
-        if constexpr (NT == 32) __syncwarp(); else __syncthreads();
-    }
-    // (a, b) summed over the group in a fixed order; every thread gets the sums
-    __device__ static void sum2(double &a, double &b, double (*red)[2])
-    {
-        for (int off = 16; off > 0; off >>= 1) {
-            a += __shfl_xor_sync(0xffffffffu, a, off);
-            b += __shfl_xor_sync(0xffffffffu, b, off);
-        }
-        if constexpr (NT > 32) {
-            if ((threadIdx.x & 31) == 0) {
-                red[threadIdx.x >> 5][0] = a;
-                red[threadIdx.x >> 5][1] = b;
-            }
-            __syncthreads();
-            double x = 0.0, y = 0.0;
-            for (int k = 0; k < NT / 32; ++k) { x += red[k][0]; y += red[k][1]; }
-            __syncthreads();
-            a = x;
-            b = y;
-        }
-    }
-};
+}  // namespace sur
+}  // namespace lbm
 
-// K*_xx and K*_yy of the leaf whose input planes start at xi; the group's work arrays hold cap cells.
-template <int NT>
-__device__ void darcy_leaf(const float *xi, int s, float *KX, float *KY, float *P, float *R, float *Dv, float *AD,
-                          double (*red)[2], double (&kd)[2])
+#include "darcy_groups.cuh"
+
+namespace lbm {
+namespace sur {
+
+// (a, b) summed over a warp in a fixed order; every lane gets the sums
+__device__ __forceinline__ void warp_sum2(double &a, double &b)
 {
-    using G = DarcyGroup<NT>;
-    const int nc = s * s, r0 = G::rank();
+    for (int off = 16; off > 0; off >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, off);
+        b += __shfl_xor_sync(0xffffffffu, b, off);
+    }
+}
+
+// K*_xx and K*_yy of the leaf whose input planes start at xi, by one warp.
+__device__ void darcy_leaf(const float *xi, int s, float *KX, float *KY, float *P, float *R, float *Dv, float *AD,
+                          double (&kd)[2])
+{
+    constexpr int NT = 32;
+    const int nc = s * s, r0 = threadIdx.x % NT;
     for (int c = r0; c < nc; c += NT) {
         const int y = c / s, xx = c - y * s;
         float v;
@@ -517,14 +498,14 @@ __device__ void darcy_leaf(const float *xi, int s, float *KX, float *KY, float *
         }
         P[c] = v;                                          // log K, for now
     }
-    G::sync();
+    __syncwarp();
     for (int c = r0; c < nc; c += NT) {
         const int y = c / s, xx = c - y * s;
         const double k = exp((double)P[c]);
         KX[c] = harmonic2f(k, exp((double)P[y * s + (xx + 1 == s ? 0 : xx + 1)]));
         KY[c] = harmonic2f(k, exp((double)P[(y + 1 == s ? 0 : y + 1) * s + xx]));
     }
-    G::sync();
+    __syncwarp();
     for (int drive = 0; drive < 2; ++drive) {
         // A p = b with (A p)_c = sum over the faces of c of k_f (p_c - p_neighbour) and
         // b_c = k_f(behind c) - k_f(ahead of c) along the drive
@@ -542,7 +523,7 @@ __device__ void darcy_leaf(const float *xi, int s, float *KX, float *KY, float *
             prz = fmaf(b, z, prz);
         }
         double rr = prr, rz = prz;
-        G::sum2(rr, rz, red);
+        warp_sum2(rr, rz);
         const double stop = 1e-10 * rr;                    // (1e-5 relative residual)^2
         for (int it = 0; it < DB_MAXIT && rr > stop; ++it) {
             float pdad = 0.0f;
@@ -557,7 +538,7 @@ __device__ void darcy_leaf(const float *xi, int s, float *KX, float *KY, float *
                 pdad = fmaf(dc, ad, pdad);
             }
             double dad = pdad, unused = 0.0;
-            G::sum2(dad, unused, red);
+            warp_sum2(dad, unused);
             if (!(dad > 0.0)) break;                          // a direction in the null space
             const float alpha = (float)(rz / dad);
             float prr2 = 0.0f, prz2 = 0.0f;
@@ -572,7 +553,7 @@ __device__ void darcy_leaf(const float *xi, int s, float *KX, float *KY, float *
                 prz2 = dg > 0.0f ? fmaf(r, r / dg, prz2) : prz2;
             }
             double rr2 = prr2, rz2 = prz2;
-            G::sum2(rr2, rz2, red);
+            warp_sum2(rr2, rz2);
             const float beta = (float)(rz2 / rz);
             rz = rz2;
             rr = rr2;
@@ -582,7 +563,7 @@ __device__ void darcy_leaf(const float *xi, int s, float *KX, float *KY, float *
                 const float dg = KX[c] + KX[cl] + KY[c] + KY[cd];
                 Dv[c] = fmaf(beta, Dv[c], dg > 0.0f ? R[c] / dg : 0.0f);
             }
-            G::sync();
+            __syncwarp();
         }
         // mean face flux along the drive
         float pq = 0.0f;
@@ -592,46 +573,30 @@ __device__ void darcy_leaf(const float *xi, int s, float *KX, float *KY, float *
                              : KY[c] * (P[c] - P[(y + 1 == s ? 0 : y + 1) * s + xx] + 1.0f);
         }
         double q = pq, unused = 0.0;
-        G::sum2(q, unused, red);
+        warp_sum2(q, unused);
         kd[drive] = q / nc;
-        G::sync();
-    }
-}
-
-// Leaves of up to 32 cells: one warp per leaf, eight warps per CTA, each with its own work arrays.
-__global__ void __launch_bounds__(DBS_WARPS * 32) darcy_small_kernel(const float *x, int n, float4 *cw)
-{
-    extern __shared__ __align__(16) unsigned char dsm_raw[];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float *base = reinterpret_cast<float *>(dsm_raw) + (size_t)w * 6 * DBS_CELLS;
-    float *KX = base, *KY = KX + DBS_CELLS, *P = KY + DBS_CELLS, *R = P + DBS_CELLS, *Dv = R + DBS_CELLS,
-          *AD = Dv + DBS_CELLS;
-    for (int i = blockIdx.x * DBS_WARPS + w; i < n; i += gridDim.x * DBS_WARPS) {
-        const float *xi = x + (int64_t)i * IN_PLANES * PIX;
-        const int s = darcy_size(xi);
-        if (s > IMG) continue;                              // the CTA kernel's leaf
-        double kd[2];
-        darcy_leaf<32>(xi, s, KX, KY, P, R, Dv, AD, nullptr, kd);
-        if (lane == 0) cw[i] = make_float4((float)log(kd[0]), 1.0f, (float)log(kd[1]), 1.0f);
         __syncwarp();
     }
 }
 
-// Leaves of 64 cells and more: one CTA per leaf.
-__global__ void __launch_bounds__(DBB_THREADS) darcy_big_kernel(const float *x, int n, float4 *cw)
+// The leaves of one list, a warp each: sides up to 3 eight warps a CTA, the sides that no leaf has but a caller's
+// size plane may say one warp a CTA, whose work arrays hold a side of 64.
+template <int WARPS, int CELLS>
+__global__ void __launch_bounds__(WARPS * 32) darcy_warp_kernel(const float *x, int n, const int *scratch, int which,
+                                                                float4 *cw)
 {
-    extern __shared__ __align__(16) unsigned char dsm_raw[];
-    float *KX = reinterpret_cast<float *>(dsm_raw);
-    float *KY = KX + DB_CELLS, *P = KY + DB_CELLS, *R = P + DB_CELLS, *Dv = R + DB_CELLS, *AD = Dv + DB_CELLS;
-    __shared__ double red[DBB_THREADS / 32][2];
-    for (int i = blockIdx.x; i < n; i += gridDim.x) {
+    extern __shared__ float dw_smem[];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float *KX = dw_smem + w * 6 * CELLS, *KY = KX + CELLS, *P = KY + CELLS, *R = P + CELLS, *Dv = R + CELLS,
+          *AD = Dv + CELLS;
+    const int *list = scratch + DG_HEADER + (int64_t)which * n;
+    for (int j = blockIdx.x * WARPS + w; j < scratch[which]; j += gridDim.x * WARPS) {
+        const int i = list[j];
         const float *xi = x + (int64_t)i * IN_PLANES * PIX;
-        const int s = darcy_size(xi);
-        if (s <= IMG) continue;                             // the warp kernel's leaf
         double kd[2];
-        darcy_leaf<DBB_THREADS>(xi, s, KX, KY, P, R, Dv, AD, red, kd);
-        if (threadIdx.x == 0) cw[i] = make_float4((float)log(kd[0]), 1.0f, (float)log(kd[1]), 1.0f);
-        __syncthreads();
+        darcy_leaf(xi, darcy_size(xi), KX, KY, P, R, Dv, AD, kd);
+        if (lane == 0) cw[i] = make_float4((float)log(kd[0]), 1.0f, (float)log(kd[1]), 1.0f);
+        __syncwarp();
     }
 }
 
@@ -659,23 +624,32 @@ __global__ void destandardise_kernel(float *y, int n, int nmodels, const float4 
 
 int nblk(int64_t n) { int64_t b = (n + 255) / 256; return (int)(b < 1 ? 1 : (b > 8192 ? 8192 : b)); }
 
-// Per-leaf target base of the given mode: patch_base_kernel (modes 0-2) or the batched Darcy
-// solve (mode 3: a warp per leaf up to 32 cells, a CTA per larger leaf).
-cudaError_t launch_base(const float *x, int n, int mode, float4 *cw, cudaStream_t st)
+// A leaf's target base and the scratch of the Darcy solves, allocated together: float4 cw[n], then ints.
+size_t base_bytes(int n) { return sizeof(float4) * (size_t)n + sizeof(int) * darcy_scratch_ints(n); }
+
+// Per-leaf target base of the given mode into cw (room for cap >= n leaves, base_bytes(cap) in all):
+// patch_base_kernel (modes 0-2) or the batched Darcy solves (mode 3).
+cudaError_t launch_base(const float *x, int n, int mode, float4 *cw, int cap, cudaStream_t st)
 {
     if (mode == 3) {
+        int *scratch = reinterpret_cast<int *>(cw + cap);
         int dev = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(darcy_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DBS_SMEM);
+            e = cudaFuncSetAttribute(darcy_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)sizeof(DarcyShared));
+        constexpr int OTHER_SMEM = 6 * DB_N * DB_N * sizeof(float), TINY_CELLS = 9;
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(darcy_big_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DBB_SMEM);
+            e = cudaFuncSetAttribute(darcy_warp_kernel<1, DB_N * DB_N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     OTHER_SMEM);
+        if (e == cudaSuccess) e = cudaMemsetAsync(scratch, 0, sizeof(int) * DG_HEADER, st);
         if (e != cudaSuccess) return e;
         const int sms = sm_count(dev);
-        const int gs = (n + DBS_WARPS - 1) / DBS_WARPS;
-        darcy_small_kernel<<<gs < sms ? gs : sms, DBS_WARPS * 32, DBS_SMEM, st>>>(x, n, cw);
-        darcy_big_kernel<<<n < 2 * sms ? n : 2 * sms, DBB_THREADS, DBB_SMEM, st>>>(x, n, cw);
-        count_launches(1);
+        darcy_classify_kernel<<<nblk(n), 256, 0, st>>>(x, n, scratch);
+        darcy_group_kernel<<<n < sms ? n : sms, RG_THREADS, sizeof(DarcyShared), st>>>(x, n, scratch, cw);
+        darcy_warp_kernel<8, TINY_CELLS><<<sms, 256, 8 * 6 * TINY_CELLS * sizeof(float), st>>>(x, n, scratch, DG_TINY, cw);
+        darcy_warp_kernel<1, DB_N * DB_N><<<2 * sms, 32, OTHER_SMEM, st>>>(x, n, scratch, DG_OTHER, cw);
+        count_launches(3);
     } else {
         patch_base_kernel<<<n < 65535 ? n : 65535, 256, 0, st>>>(x, n, mode, cw);
     }
@@ -1208,8 +1182,8 @@ lbm_status lbm_surrogate_predict(lbm_surrogate *s, const float *x_dev, int32_t n
         }
     }
     float4 *d_cw = nullptr;
-    SUR_CUDA(cudaMalloc(&d_cw, sizeof(float4) * n));
-    cudaError_t eb = launch_base(x_dev, n, s->target_mode, d_cw, st);
+    SUR_CUDA(cudaMalloc(&d_cw, base_bytes(n)));
+    cudaError_t eb = launch_base(x_dev, n, s->target_mode, d_cw, n, st);
     if (eb != cudaSuccess) {
         cudaFree(d_cw);
         cudaGetLastError();
@@ -1247,8 +1221,8 @@ lbm_status lbm_surrogate_train(lbm_surrogate *s, const float *x_dev, const float
     std::vector<float> cw((size_t)4 * n);
     {
         float4 *d_cw = nullptr;
-        SUR_CUDA(cudaMalloc(&d_cw, sizeof(float4) * n));
-        cudaError_t e1 = launch_base(x_dev, n, s->target_mode, d_cw, st);
+        SUR_CUDA(cudaMalloc(&d_cw, base_bytes(n)));
+        cudaError_t e1 = launch_base(x_dev, n, s->target_mode, d_cw, n, st);
         if (e1 == cudaSuccess) e1 = cudaMemcpy(cw.data(), d_cw, sizeof(float4) * n, cudaMemcpyDeviceToHost);
         cudaFree(d_cw);
         if (e1 != cudaSuccess) { cudaGetLastError(); return fail(LBM_ECUDA, "patch bases: %s", cudaGetErrorString(e1)); }
@@ -1498,7 +1472,7 @@ static lbm_status ensure_keff_work(lbm_surrogate *s, int chunk, int64_t n)
         e = cudaMalloc(&s->kx, sizeof(float) * (size_t)chunk * IN_PLANES * PIX);
         if (e == cudaSuccess) e = cudaMalloc(&s->kstats, sizeof(float) * (size_t)chunk * 3);
         if (e == cudaSuccess) e = cudaMalloc(&s->ky, sizeof(float) * (size_t)chunk * 2 * s->nmodels);
-        if (e == cudaSuccess) e = cudaMalloc(&s->kcw, sizeof(float4) * (size_t)chunk);
+        if (e == cudaSuccess) e = cudaMalloc(&s->kcw, base_bytes(chunk));
         if (e == cudaSuccess) s->kcap = chunk;
     }
     if (e == cudaSuccess && n > s->jcap) {
@@ -1599,7 +1573,7 @@ lbm_status lbm_surrogate_keff(lbm_surrogate *s, const lbm_params *p, const float
                                          cudaMemcpyDeviceToDevice, st));
             }
         }
-        SUR_CUDA(launch_base(s->kx, nc, s->target_mode, s->kcw, st));
+        SUR_CUDA(launch_base(s->kx, nc, s->target_mode, s->kcw, s->kcap, st));
         destandardise_kernel<<<nblk((int64_t)s->nmodels * nc * 2), 256, 0, st>>>(
             s->ky, nc, s->nmodels, s->kcw, s->y_mean[0], s->y_std[0], s->y_mean[1], s->y_std[1]);
         gate_kernel<<<nblk(nc), 256, 0, st>>>(s->ky, s->nmodels, nc, b0, lv, s->kstats, ga, keff_dev, fb, s->table);

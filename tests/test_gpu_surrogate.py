@@ -387,3 +387,22 @@ def test_gate_routes_blocks():
     np.testing.assert_allclose(ks[:, 0], np.exp(pred[:, :, 0].sum(axis=0) / 3), rtol=1e-15)
     np.testing.assert_allclose(ks[:, 3], np.exp(pred[:, :, 1].sum(axis=0) / 3), rtol=1e-15)
     assert (ks[:, 1] == 0).all() and (ks[:, 2] == 0).all()
+
+
+@pytest.mark.parametrize("counts", [{4: 35, 8: 9, 2: 5, 1: 3}, {64: 2, 32: 5, 16: 3, 8: 1, 4: 1}, {16: 400}])
+def test_darcy_base_of_every_side_matches_oracle(counts):
+    """The Darcy base (mode 3) groups leaves by side: a part of a warp to sixteen warps each, batches
+    that do not fill a warp's places, and more leaves than groups. 3e-5 is the bound of the test above."""
+    lbm = _lbm()
+    rng = np.random.default_rng(17)
+    leaves = []
+    for s, n in counts.items():
+        for i in range(n):
+            z = synth.gaussian_random_field(s, s, 2.0, seed=100 * s + i) if s > 1 else np.zeros((1, 1))
+            leaves.append(rng.normal(-4.0, 1.0) + 1.0 * z)
+    leaves = [leaves[i] for i in rng.permutation(len(leaves))]
+    x = _inputs(len(leaves), 0, leaves)
+    with lbm.Surrogate(1, 0) as sur:
+        c, _ = _base_from_predict(sur, x, 3)
+    ref = np.array([S.target_base(lk.astype(np.float32).astype(np.float64), 3) for lk in leaves])
+    np.testing.assert_allclose(c, ref[:, [0, 2]], rtol=0, atol=3e-5)
