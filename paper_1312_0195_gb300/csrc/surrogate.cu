@@ -10,6 +10,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 namespace lbm {
@@ -110,28 +111,32 @@ __global__ void __launch_bounds__(256) patch_kernel(const float *kappa, int nx, 
         p[q] = 0.25f * ((v[0] + v[1]) + (v[2] + v[3]));
     }
     __syncthreads();
-    // context planes: harmonic and arithmetic means of K = exp(p) along each row and each column
-    __shared__ double rk[IMG], ri[IMG], ck[IMG], ci[IMG];
-    if (threadIdx.x < IMG) {
-        const int r = threadIdx.x;
-        double a = 0.0, b = 0.0;
-        for (int c = 0; c < IMG; ++c) { a += exp((double)p[r * IMG + c]); b += exp(-(double)p[r * IMG + c]); }
-        rk[r] = a;
-        ri[r] = b;
-    } else if (threadIdx.x < 2 * IMG) {
-        const int c = threadIdx.x - IMG;
-        double a = 0.0, b = 0.0;
-        for (int r = 0; r < IMG; ++r) { a += exp((double)p[r * IMG + c]); b += exp(-(double)p[r * IMG + c]); }
-        ck[c] = a;
-        ci[c] = b;
+    // context planes: harmonic and arithmetic means of K = exp(p) along each row and each column. Each
+    // pixel's two exponentials and each line's logarithm are taken once (FP64 is slow here: taken where they
+    // are used, 4096 + 4096 a leaf, they were most of this kernel's time, 0.38 us a leaf against 0.10)
+    __shared__ double ke[IMG][IMG + 1], ie[IMG][IMG + 1];
+    __shared__ float line[4][IMG];
+    for (int q = threadIdx.x; q < PIX; q += blockDim.x) {
+        ke[q >> 5][q & 31] = exp((double)p[q]);
+        ie[q >> 5][q & 31] = exp(-(double)p[q]);
+    }
+    __syncthreads();
+    if (threadIdx.x < 4 * IMG) {
+        const int which = threadIdx.x >> 5, i = threadIdx.x & 31;    // 1 / K then K along a row, then a column
+        double a = 0.0;
+        for (int j = 0; j < IMG; ++j) {
+            const int r = which < 2 ? i : j, c = which < 2 ? j : i;
+            a += (which & 1) ? ke[r][c] : ie[r][c];
+        }
+        line[which][i] = (which & 1) ? (float)log(a / IMG) : (float)(-log(a / IMG));
     }
     __syncthreads();
     for (int q = threadIdx.x; q < PIX; q += blockDim.x) {
         const int py = q >> 5, px = q & 31;
-        xi[5 * PIX + q] = (float)(-log(ri[py] / IMG));
-        xi[6 * PIX + q] = (float)log(rk[py] / IMG);
-        xi[7 * PIX + q] = (float)(-log(ci[px] / IMG));
-        xi[8 * PIX + q] = (float)log(ck[px] / IMG);
+        xi[5 * PIX + q] = line[0][py];
+        xi[6 * PIX + q] = line[1][py];
+        xi[7 * PIX + q] = line[2][px];
+        xi[8 * PIX + q] = line[3][px];
     }
     double sm = 0.0, sq = 0.0, ge = 0.0;
     for (int q = threadIdx.x; q < PIX; q += blockDim.x) {
@@ -182,30 +187,29 @@ __global__ void __launch_bounds__(256) input_kernel(const float *x, const int *i
     }
 }
 
-// B operand of the forward conv: row n = c_out, k = tap * CIN_P + c_in.
-__global__ void pack_fwd_kernel(const float *w, int cin, int cin_p, int cout, __nv_bfloat16 *out)
-{
-    const int K = 9 * cin_p;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < cout * K; t += gridDim.x * blockDim.x) {
-        const int n = t / K, k = t - n * K, tap = k / cin_p, ci = k - tap * cin_p;
-        const float v = ci < cin ? w[((int64_t)n * cin + ci) * 9 + tap] : 0.0f;
-        out[umma::core_offset(n, k, K) / 2] = __float2bfloat16_rn(v);
-    }
-}
-
-// B operand of the input-gradient conv: row n = c_in, k = tap' * COUT + c_out, value
+// The tensor-core operands of one model's convolutions, every layer in one launch (block row y):
+// y < NLAYER: the forward conv's B operand, row n = c_out, k = tap * CIN_P + c_in;
+// y >= NLAYER: the input-gradient conv's of layer y - NLAYER + 1, row n = c_in, k = tap' * COUT + c_out, value
 // W[c_out][c_in][8 - tap'] (the transposed, spatially flipped kernel).
-__global__ void pack_bwd_kernel(const float *w, int cin, int cout, __nv_bfloat16 *out)
+struct PackArgs {
+    const float *w[NLAYER];
+    __nv_bfloat16 *fwd[NLAYER], *bwd[NLAYER];
+};
+__global__ void __launch_bounds__(256) pack_kernel(PackArgs a)
 {
-    const int K = 9 * cout;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < cin * K; t += gridDim.x * blockDim.x) {
-        const int n = t / K, k = t - n * K, tp = k / cout, co = k - tp * cout;
-        out[umma::core_offset(n, k, K) / 2] = __float2bfloat16_rn(w[((int64_t)co * cin + n) * 9 + (8 - tp)]);
-    }
+    const bool back = blockIdx.y >= NLAYER;
+    const int l = back ? blockIdx.y - NLAYER + 1 : blockIdx.y;
+    const int cin = cin_real(l), cout = cout_of(l), depth = back ? cout : cin_p(l), rows = back ? cin : cout;
+    const int K = 9 * depth, t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= rows * K) return;
+    const int n = t / K, k = t - n * K, tap = k / depth, c = k - tap * depth;
+    const float v = back ? a.w[l][((int64_t)c * cin + n) * 9 + (8 - tap)]
+                         : (c < cin ? a.w[l][((int64_t)n * cin + c) * 9 + tap] : 0.0f);
+    (back ? a.bwd[l] : a.fwd[l])[umma::core_offset(n, k, K) / 2] = __float2bfloat16_rn(v);
 }
 
-// Global average pooling of the last activation and the linear head. One CTA per image;
-// thread t reads elements t, t + 256, ... of each 8-channel plane (always channel t % 8), and
+// Global average pooling of the last activation and the linear head. One CTA per image; a warp
+// takes an 8-channel plane, lane l the pixels l, l + 32, ... (16 bytes, all eight channels), and
 // the 32 partial sums of a channel are folded in a fixed order.
 __global__ void __launch_bounds__(256) gap_head_kernel(const __nv_bfloat16 *act, const float *wh, const float *bh,
                                                       float *pooled, float *y)
@@ -213,11 +217,19 @@ __global__ void __launch_bounds__(256) gap_head_kernel(const __nv_bfloat16 *act,
     const int b = blockIdx.x, t = threadIdx.x;
     __shared__ float part[32][64];
     __shared__ float pool[64];
-    for (int g = 0; g < 8; ++g) {
-        const __nv_bfloat16 *plane = act + act_at(b, 0, 8 * g, 64);
-        float s = 0.0f;
-        for (int e = t; e < PIX * 8; e += 256) s += __bfloat162float(plane[e]);
-        part[t >> 3][8 * g + (t & 7)] = s;
+    {
+        const int g = t >> 5, l = t & 31;
+        const uint4 *plane = reinterpret_cast<const uint4 *>(act + act_at(b, 0, 8 * g, 64));
+        float s[8] = {};
+#pragma unroll 16
+        for (int p = l; p < PIX; p += 32) {
+            const uint4 in = plane[p];
+            const __nv_bfloat16 *v = reinterpret_cast<const __nv_bfloat16 *>(&in);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) s[c] += __bfloat162float(v[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) part[l][8 * g + c] = s[c];
     }
     __syncthreads();
     if (t < 64) {
@@ -235,66 +247,136 @@ __global__ void __launch_bounds__(256) gap_head_kernel(const __nv_bfloat16 *act,
     }
 }
 
-// Loss L = mean((y - t)^2) over B x 2 entries (targets already standardised), the head's
-// gradients and dL/dpool. One CTA; every sum runs in a fixed order.
-__global__ void __launch_bounds__(256) loss_head_backward_kernel(const float *y, const float *t, const float *pooled,
-                                                                const float *wh, int B, float *dpool, float *gwh,
-                                                                float *gbh, float *loss)
+// Copies to shared memory that stay in flight while the thread goes on: sums that must be taken in order wait
+// for memory once per batch of them, not once per term (the compiler sinks plain loads to their adds).
+template <int BYTES> __device__ __forceinline__ void copy_ahead(void *dst, const void *src)
 {
-    __shared__ float dy[2][1024];
-    for (int b = threadIdx.x; b < B; b += blockDim.x) {
-        dy[0][b] = 2.0f * (y[2 * b] - t[2 * b]) / (2.0f * B);
-        dy[1][b] = 2.0f * (y[2 * b + 1] - t[2 * b + 1]) / (2.0f * B);
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(umma::smem_addr(dst)), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(umma::smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int LEFT> __device__ __forceinline__ void copies_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory");
+}
+
+// Loss L = mean((y - t)^2) over B x 2 entries (targets already standardised), the head's
+// gradients and dL/dpool. Block 0 takes the sums over the batch (every one in a fixed order, loads batched
+// ahead of it), the others dL/dpool.
+constexpr int LOSS_THREADS = 256, LOSS_IMGS = 16;            // images of a block's dL/dpool
+__global__ void __launch_bounds__(LOSS_THREADS) loss_head_backward_kernel(const float *y, const float *t,
+                                                                         const float *pooled, const float *wh, int B,
+                                                                         float *dpool, float *gwh, float *gbh,
+                                                                         float *loss)
+{
+    auto dy_of = [&](int b, int o) { return 2.0f * (y[2 * b + o] - t[2 * b + o]) / (2.0f * B); };
+    if (blockIdx.x > 0) {
+        const int b0 = (blockIdx.x - 1) * LOSS_IMGS;
+        for (int q = threadIdx.x; q < LOSS_IMGS * 64; q += LOSS_THREADS) {
+            const int b = b0 + (q >> 6), c = q & 63;
+            if (b < B) dpool[(int64_t)b * 64 + c] = dy_of(b, 0) * wh[c] + dy_of(b, 1) * wh[64 + c];
+        }
+        return;
     }
+    __shared__ float dy[2][1024];
+    __shared__ double part[LOSS_THREADS / 32];
+    double sq = 0.0;
+    for (int b = threadIdx.x; b < B; b += LOSS_THREADS) {
+        dy[0][b] = dy_of(b, 0);
+        dy[1][b] = dy_of(b, 1);
+        const double e0 = (double)y[2 * b] - t[2 * b], e1 = (double)y[2 * b + 1] - t[2 * b + 1];
+        sq += e0 * e0 + e1 * e1;
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = sq;
     __syncthreads();
     if (threadIdx.x < 128) {
         const int o = threadIdx.x >> 6, c = threadIdx.x & 63;
+        constexpr int BATCH = 64;
         float acc = 0.0f;
-        for (int b = 0; b < B; ++b) acc += dy[o][b] * pooled[(int64_t)b * 64 + c];
+        int b = 0;
+        for (; b + BATCH <= B; b += BATCH) {
+            float v[BATCH];
+#pragma unroll
+            for (int u = 0; u < BATCH; ++u) v[u] = pooled[(int64_t)(b + u) * 64 + c];
+#pragma unroll
+            for (int u = 0; u < BATCH; ++u) acc = fmaf(dy[o][b + u], v[u], acc);
+        }
+        for (; b < B; ++b) acc = fmaf(dy[o][b], pooled[(int64_t)b * 64 + c], acc);
         gwh[o * 64 + c] = acc;
     } else if (threadIdx.x < 130) {
         const int o = threadIdx.x - 128;
         float acc = 0.0f;
+#pragma unroll 16
         for (int b = 0; b < B; ++b) acc += dy[o][b];
         gbh[o] = acc;
-    } else if (threadIdx.x == 130) {
+    } else if (threadIdx.x == 160) {
         double acc = 0.0;
-        for (int b = 0; b < B; ++b) {
-            const double e0 = (double)y[2 * b] - t[2 * b], e1 = (double)y[2 * b + 1] - t[2 * b + 1];
-            acc += e0 * e0 + e1 * e1;
-        }
+        for (int w = 0; w < LOSS_THREADS / 32; ++w) acc += part[w];
         *loss = (float)(acc / (2.0 * B));
-    }
-    for (int q = threadIdx.x; q < B * 64; q += blockDim.x) {
-        const int b = q >> 6, c = q & 63;
-        dpool[q] = dy[0][b] * wh[c] + dy[1][b] * wh[64 + c];
     }
 }
 
-// dL/d(last activation), ReLU mask applied: dpool / 1024 where the activation is positive.
+// dL/d(last activation), ReLU mask applied: dpool / 1024 where the activation is positive. A thread takes a
+// pixel's eight channels (16 bytes).
 __global__ void __launch_bounds__(256) gap_backward_kernel(const float *dpool, const __nv_bfloat16 *act, int B,
                                                           __nv_bfloat16 *dact)
 {
-    const int64_t total = (int64_t)B * PIX * 64;
+    const int64_t total = (int64_t)B * 8 * PIX;              // act_at layout: [B][8 groups][PIX][8]
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t b = t / (PIX * 64);
-        const int c = (int)((t / (PIX * 8)) & 7) * 8 + (int)(t & 7);      // act_at layout
-        const float g = __bfloat162float(act[t]) > 0.0f ? dpool[b * 64 + c] / PIX : 0.0f;
-        dact[t] = __float2bfloat16_rn(g);
+        const uint4 in = reinterpret_cast<const uint4 *>(act)[t];
+        const __nv_bfloat16 *a = reinterpret_cast<const __nv_bfloat16 *>(&in);
+        const float *d = dpool + (t / PIX) * 8;              // channels 8 g .. 8 g + 7 of image b, t / PIX = 8 b + g
+        uint4 out;
+        __nv_bfloat16 *o = reinterpret_cast<__nv_bfloat16 *>(&out);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) o[c] = __float2bfloat16_rn(__bfloat162float(a[c]) > 0.0f ? d[c] / PIX : 0.0f);
+        reinterpret_cast<uint4 *>(dact)[t] = out;
     }
 }
 
 // Bias gradient partials: bpart[g][co] = sum over images g, g + G, ... and all their pixels of
 // dout[img][p][co] (dout holds the ReLU-masked gradient of the layer's output). Thread t sums
-// channel t % COUT over pixels p = t / COUT (mod 256 / COUT); the phases are folded in order.
+// channel t % COUT over pixels p = t / COUT (mod 256 / COUT) in order; the phases are folded in order. Half
+// images are copied to shared memory one ahead of the sums (planes 16 bytes apart modulo the banks, so a warp's
+// four planes do not collide): 9 us for 256 images of 64 channels, 25 with loads from global memory.
+constexpr int BG_PIX = PIX / 2;
+constexpr int BG_PLANE = BG_PIX * 8 + 8;                     // elements of a staged plane
+template <int COUT> constexpr size_t bg_smem() { return 2 * (COUT / 8) * BG_PLANE * sizeof(__nv_bfloat16); }
 template <int COUT>
 __global__ void __launch_bounds__(256) bias_grad_kernel(const __nv_bfloat16 *dout, int B, float *bpart)
 {
-    constexpr int NPH = 256 / COUT;
+    constexpr int NPH = 256 / COUT, G = COUT / 8;
+    extern __shared__ __align__(16) unsigned char bg_raw[];
+    __nv_bfloat16 *stage = reinterpret_cast<__nv_bfloat16 *>(bg_raw);
     const int t = threadIdx.x, co = t % COUT, ph = t / COUT;
+    const int n = 2 * ((B - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x);     // half images of this CTA
+    auto fetch = [&](int h) {
+        if (h < n) {
+            const int img = blockIdx.x + (h >> 1) * gridDim.x;
+            const __nv_bfloat16 *src = dout + act_at(img, (h & 1) * BG_PIX, 0, COUT);
+            __nv_bfloat16 *dst = stage + (h & 1) * G * BG_PLANE;
+            for (int q = t; q < G * BG_PIX; q += 256) {
+                const int g = q / BG_PIX, p = q - g * BG_PIX;
+                copy_ahead<16>(dst + g * BG_PLANE + p * 8, src + (int64_t)g * PIX * 8 + p * 8);
+            }
+        }
+        copies_commit();
+    };
+    fetch(0);
     float acc = 0.0f;
-    for (int img = blockIdx.x; img < B; img += gridDim.x)
-        for (int p = ph; p < PIX; p += NPH) acc += __bfloat162float(dout[act_at(img, p, co, COUT)]);
+    for (int h = 0; h < n; ++h) {
+        fetch(h + 1);
+        copies_wait<1>();
+        __syncthreads();
+        const __nv_bfloat16 *src = stage + (h & 1) * G * BG_PLANE + (co >> 3) * BG_PLANE + (co & 7);
+#pragma unroll 16
+        for (int p = ph; p < BG_PIX; p += NPH) acc += __bfloat162float(src[p * 8]);
+        __syncthreads();
+    }
     __shared__ float red[256];
     red[t] = acc;
     __syncthreads();
@@ -307,27 +389,52 @@ __global__ void __launch_bounds__(256) bias_grad_kernel(const __nv_bfloat16 *dou
 
 // Folds the per-CTA partials of wgrad_tc_kernel (CTA b holds input-channel part b % P; its rows h
 // are separate partials) into W's gradient [co][ci][3][3] and the bias partials into b's, in a
-// fixed order (deterministic).
-__global__ void __launch_bounds__(256) wgrad_tc_reduce_kernel(const float *part, int grid, int P, int HM, int cout,
-                                                             int cip, int cin, const float *bpart, int nb, float *gw,
-                                                             float *gb)
+// fixed order (deterministic). A thread owns one element of the partials' own layout [tap][co][c], so a warp
+// copies whole lines, RED_ROWS of them in flight, and adds its own in order from shared memory. The fold is bound by
+// those copies (22 MB at 64 -> 64 channels); threads that followed the order of W and waited for each load
+// took 75 us at 64 -> 64 and 32 -> 32 channels, these 11 and 21.
+constexpr int RED_ROWS = 76, RED_THREADS = 128;
+constexpr size_t RED_SMEM = 2 * (size_t)RED_ROWS * RED_THREADS * sizeof(float);
+template <int HM>
+__global__ void __launch_bounds__(RED_THREADS) wgrad_tc_reduce_kernel(const float *part, int grid, int P, int cout,
+                                                                     int cip, int cin, const float *bpart, int nb,
+                                                                     float *gw, float *gb)
 {
-    const int nw = cout * cin * 9;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nw + cout; t += gridDim.x * blockDim.x) {
-        if (t < nw) {
-            const int co = t / (cin * 9), rem = t - co * cin * 9, ci = rem / 9, tap = rem - ci * 9;
-            const int pp = ci / cip, c = ci - pp * cip;
-            float acc = 0.0f;
-            for (int b = pp; b < grid; b += P)
-                for (int h = 0; h < HM; ++h)
-                    acc += part[((((int64_t)b * HM + h) * 9 + tap) * cout + co) * cip + c];
-            gw[t] = acc;
-        } else {
-            const int co = t - nw;
-            float acc = 0.0f;
-            for (int b = 0; b < nb; ++b) acc += bpart[(int64_t)b * cout + co];
-            gb[co] = acc;
+    extern __shared__ float red_smem[];
+    const int per = 9 * cout * cip, nw = P * per;            // elements of a partial row; of all parts
+    // src[(k / H) * step + (k % H) * per] for k = 0 .. n - 1, summed in that order
+    auto fold = [&](const float *src, int n, int64_t step, auto rows) {
+        constexpr int H = decltype(rows)::value;
+        float *mine = red_smem + threadIdx.x;
+        auto fetch = [&](int k0) {
+            float *dst = mine + (k0 / RED_ROWS & 1) * RED_ROWS * RED_THREADS;
+            for (int k = k0; k < min(k0 + RED_ROWS, n); ++k)
+                copy_ahead<4>(dst + (k - k0) * RED_THREADS, src + (k / H) * step + (int64_t)(k % H) * per);
+            copies_commit();
+        };
+        fetch(0);
+        float acc = 0.0f;
+        for (int k0 = 0; k0 < n; k0 += RED_ROWS) {
+            fetch(k0 + RED_ROWS);
+            copies_wait<1>();                                // a thread reads only what it copied itself
+            const float *v = mine + (k0 / RED_ROWS & 1) * RED_ROWS * RED_THREADS;
+            const int m = min(RED_ROWS, n - k0);
+#pragma unroll 8
+            for (int k = 0; k < m; ++k) acc += v[k * RED_THREADS];
         }
+        copies_wait<0>();
+        return acc;
+    };
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < nw) {
+        const int pp = t / per, e = t - pp * per;
+        const int tap = e / (cout * cip), co = (e / cip) % cout, ci = pp * cip + e % cip;
+        if (ci >= cin) return;                               // padded input channels
+        // CTAs pp, pp + P, ... in order, the HM rows of each in turn
+        gw[((int64_t)co * cin + ci) * 9 + tap] = fold(part + (int64_t)pp * HM * per + e, (grid - pp + P - 1) / P * HM,
+                                                      (int64_t)P * HM * per, std::integral_constant<int, HM>{});
+    } else if (t < nw + cout) {
+        gb[t - nw] = fold(bpart + (t - nw), nb, cout, std::integral_constant<int, 1>{});
     }
 }
 
@@ -793,6 +900,12 @@ static cudaError_t launch_wgrad_tc(const __nv_bfloat16 *in, const __nv_bfloat16 
         const cudaError_t e = cudaFuncSetAttribute(wgrad_tc_kernel<COUT, CIN_P, CIP>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W::SMEM);
         if (e != cudaSuccess) return e;
+        const cudaError_t e2 = cudaFuncSetAttribute(wgrad_tc_reduce_kernel<W::HM>,
+                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RED_SMEM);
+        if (e2 != cudaSuccess) return e2;
+        const cudaError_t e3 = cudaFuncSetAttribute(bias_grad_kernel<COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                    (int)bg_smem<COUT>());
+        if (e3 != cudaSuccess) return e3;
         sms = sm_count(dev);
     }
     CUtensorMap tin, tout;
@@ -805,9 +918,10 @@ static cudaError_t launch_wgrad_tc(const __nv_bfloat16 *in, const __nv_bfloat16 
     WgtArgs a{part, B, err};
     wgrad_tc_kernel<COUT, CIN_P, CIP><<<grid, CONV_THREADS, W::SMEM, st>>>(tin, tout, a);
     const int nb = B < 128 ? B : 128;
-    bias_grad_kernel<COUT><<<nb, 256, 0, st>>>(dout, B, bpart);
-    wgrad_tc_reduce_kernel<<<nblk((int64_t)COUT * cin * 9 + COUT), 256, 0, st>>>(part, grid, W::P, W::HM, COUT, CIP,
-                                                                                cin, bpart, nb, gw, gb);
+    bias_grad_kernel<COUT><<<nb, 256, bg_smem<COUT>(), st>>>(dout, B, bpart);
+    constexpr int elements = 9 * COUT * CIN_P + COUT;
+    wgrad_tc_reduce_kernel<W::HM><<<(elements + RED_THREADS - 1) / RED_THREADS, RED_THREADS, RED_SMEM, st>>>(
+        part, grid, W::P, COUT, CIP, cin, bpart, nb, gw, gb);
     count_launches(3);
     return cudaGetLastError();
 }
@@ -932,12 +1046,15 @@ static lbm_status ensure_work(lbm_surrogate *s, int B)
 static cudaError_t pack_model(lbm_surrogate *s, int m, cudaStream_t st)
 {
     const float *P = s->params + (int64_t)m * LAYOUT.total;
+    PackArgs a;
     for (int l = 0; l < NLAYER; ++l) {
-        const int ci = cin_real(l), cp = cin_p(l), co = cout_of(l);
-        pack_fwd_kernel<<<nblk((int64_t)co * 9 * cp), 256, 0, st>>>(P + LAYOUT.w[l], ci, cp, co, s->wf[l]);
-        if (l >= 1) pack_bwd_kernel<<<nblk((int64_t)ci * 9 * co), 256, 0, st>>>(P + LAYOUT.w[l], ci, co, s->wb[l]);
+        a.w[l] = P + LAYOUT.w[l];
+        a.fwd[l] = s->wf[l];
+        a.bwd[l] = s->wb[l];
     }
-    count_launches(2 * NLAYER - 1);
+    const dim3 blocks((64 * 9 * 64 + 255) / 256, 2 * NLAYER - 1);    // the largest layer's operand
+    pack_kernel<<<blocks, 256, 0, st>>>(a);
+    count_launches(1);
     return cudaGetLastError();
 }
 
@@ -960,9 +1077,9 @@ static cudaError_t backward(lbm_surrogate *s, int m, int B, cudaStream_t st)
 {
     const float *P = s->params + (int64_t)m * LAYOUT.total;
     float *G = s->grad;
-    loss_head_backward_kernel<<<1, 256, 0, st>>>(s->y, s->t, s->pooled, P + LAYOUT.wh, B, s->dpool, G + LAYOUT.wh,
+    loss_head_backward_kernel<<<1 + (B + LOSS_IMGS - 1) / LOSS_IMGS, LOSS_THREADS, 0, st>>>(s->y, s->t, s->pooled, P + LAYOUT.wh, B, s->dpool, G + LAYOUT.wh,
                                                  G + LAYOUT.bh, s->loss);
-    gap_backward_kernel<<<nblk((int64_t)B * PIX * 64), 256, 0, st>>>(s->dpool, s->act[NLAYER], B, s->dact[0]);
+    gap_backward_kernel<<<nblk((int64_t)B * PIX * 8), 256, 0, st>>>(s->dpool, s->act[NLAYER], B, s->dact[0]);
     count_launches(2);
     int cur = 0;
     for (int l = NLAYER - 1; l >= 0; --l) {
