@@ -625,6 +625,22 @@ template <> __device__ __forceinline__ double ld_cluster<double>(uint32_t a)
     asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a));
     return v;
 }
+template <> __device__ __forceinline__ float2 ld_cluster<float2>(uint32_t a)
+{
+    float2 v;
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void st_cluster(uint32_t a, float2 v)
+{
+    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y));
+}
+template <> __device__ __forceinline__ int ld_cluster<int>(uint32_t a)
+{
+    int v;
+    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
 __device__ __forceinline__ void st_cluster(uint32_t a, float v)
 {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v));
@@ -899,6 +915,14 @@ __global__ void __launch_bounds__(clu3_threads<T>(), 1) local3d_cluster_kernel(C
     cluster_sync_all();     // no CTA leaves while a peer may still read its shared memory
 }
 
+}  // namespace
+}  // namespace lbm
+
+#include "local3_pair.cuh"
+
+namespace lbm {
+namespace {
+
 // The compiled slot strides: FP32 up to 2048 cells per slab, FP64 up to 1024
 template <typename T>
 const void *clu3_kernel(int ps)
@@ -918,6 +942,16 @@ const void *clu3_kernel(int ps)
 inline size_t clu3_smem_bytes(int64_t PS, size_t esz)
 {
     return sizeof(double) * (4 + 96 + 16) + (size_t)PS * Q19 * esz;
+}
+
+const void *pair3_kernel(int ps)
+{
+    switch (ps) {
+    case 256: return reinterpret_cast<const void *>(&local3d_pair_kernel<256>);
+    case 512: return reinterpret_cast<const void *>(&local3d_pair_kernel<512>);
+    case 1024: return reinterpret_cast<const void *>(&local3d_pair_kernel<1024>);
+    default: return nullptr;
+    }
 }
 
 // e per cell of every job of a chunk: job j copies its leaf's cube of the field
@@ -1035,6 +1069,89 @@ void free3(lbm3d_grid *g)
 
 namespace {
 
+// After the launches of one leaf size: the wall-clock limit's verdict.
+lbm_status cluster_result(const unsigned long long *d_clock, cudaStream_t st)
+{
+    unsigned long long clk[2] = {0, 0};
+    if (cudaMemcpyAsync(clk, d_clock, sizeof(clk), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(LBM_ECUDA, "local problems failed on the device");
+    }
+    if (reinterpret_cast<const int *>(&clk[1])[0])
+        return fail(LBM_ETIMEOUT, "local problems exceeded the time limit; unfinished leaves carry LBM_ETIMEOUT");
+    return LBM_OK;
+}
+
+// The same two jobs at a time (local3_pair.cuh): FP32 cubes of at most CP3_MAX_SIDE cells a side, whose slabs take
+// clusters of at most 6 CTAs. LBM_EINVAL (nothing launched) for other cubes, or if the device cannot schedule
+// such a cluster. Measured on batches that fill the chip, billions of updates a second, one job a cluster -> two:
+// side 8 136 -> 160, 10 118 -> 122, 12 98 -> 122, 14 91 -> 97, 16 109 -> 120, 18 78 -> 97.
+lbm_status run_pair_size(const lbm3d_params *p, const float *kappa_dev, const int4 *d_l4, const std::vector<int> &ids,
+                         int *d_ids, int sz, int m, double nu, double g_const, double tol_rel, int64_t max_steps,
+                         int32_t check_every, int optin, unsigned long long *d_clock, double *keff_dev,
+                         int32_t *status_dev, int32_t *steps_dev, cudaStream_t st)
+{
+    if (p->storage != LBM_F32 || sz > CP3_MAX_SIDE || ids.size() > (size_t)INT_MAX / 3 - 1) return LBM_EINVAL;
+    const int s2 = sz * sz;
+    int C = 0, L = 0;
+    // slabs of at most 512 cells (two CTAs on an SM cover each other's barriers) where they take at most 4 CTAs,
+    // else of at most 1024 (side 12: 122 against 111 billion updates a second; 16, with 8 CTAs: 103 against 120)
+    for (int cells : {512, CP3_THREADS * CP3_CPT}) {
+        const int lmax = std::max(1, cells / s2), c = (sz + lmax - 1) / lmax;
+        L = (sz + c - 1) / c;
+        C = (sz + L - 1) / L;
+        if (C <= 4) break;
+    }
+    const int P = L * s2;
+    const int PS = P <= 256 ? 256 : (P <= 512 ? 512 : 1024);
+    const size_t smem = pair3_smem_bytes(PS);
+    const void *fn = pair3_kernel(PS);
+    if (smem > (size_t)optin) return LBM_EINVAL;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+        cudaGetLastError();
+        return LBM_EINVAL;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.blockDim = dim3((unsigned)std::min(CP3_THREADS, ((P + CP3_CPT - 1) / CP3_CPT + 31) / 32 * 32));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cfg.gridDim = dim3((unsigned)C);
+    int nclusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) != cudaSuccess || nclusters < 1) {
+        cudaGetLastError();
+        return LBM_EINVAL;
+    }
+    const int n = (int)ids.size(), njobs = 3 * n;
+    int *head = reinterpret_cast<int *>(d_clock + 2);
+    if (cudaMemcpyAsync(d_ids, ids.data(), sizeof(int) * n, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+        cudaMemsetAsync(head, 0, sizeof(int), st) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(LBM_ECUDA, "copying the leaf list failed");
+    }
+    cfg.gridDim = dim3((unsigned)(C * std::min(nclusters, (njobs + 1) / 2)));
+    Clu3Args<float> a{kappa_dev, p->nx, p->ny, p->nz, d_l4, d_ids, njobs, sz, L, m, (float)(1.0 / p->tau),
+                      (float)(6.0 * p->tau), (float)(3.0 * (1.0 - 2.0 * p->tau)), (float)(0.5 * p->eps * g_const),
+                      p->eps * nu, nu / g_const, tol_rel, check_every, max_steps, keff_dev, status_dev,
+                      steps_dev, d_clock, reinterpret_cast<int *>(d_clock + 1),
+                      (unsigned long long)(local_time_limit() * 1e9)};
+    void *args[] = {&a, &head};
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
+    count_launches(1);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return fail(LBM_ECUDA, "cluster launch failed: %s", cudaGetErrorString(e));
+    }
+    return cluster_result(d_clock, st);
+}
+
 // Runs every job of one leaf size on the cluster path. Returns LBM_EINVAL (nothing
 // launched) when the cube does not fit the shared memory of a cluster of at most 16
 // CTAs or the device cannot schedule such a cluster.
@@ -1128,15 +1245,7 @@ lbm_status run_cluster_size(const lbm3d_params *p, const float *kappa_dev, const
             return fail(LBM_ECUDA, "cluster launch failed: %s", cudaGetErrorString(e));
         }
     }
-    unsigned long long clk[2] = {0, 0};
-    if (cudaMemcpyAsync(clk, d_clock, sizeof(clk), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(LBM_ECUDA, "local problems failed on the device");
-    }
-    if (reinterpret_cast<const int *>(&clk[1])[0])
-        return fail(LBM_ETIMEOUT, "local problems exceeded the time limit; unfinished leaves carry LBM_ETIMEOUT");
-    return LBM_OK;
+    return cluster_result(d_clock, st);
 }
 
 }  // namespace
@@ -1469,7 +1578,7 @@ lbm_status lbm3d_local_keff_batch(const lbm3d_params *p, const float *kappa_dev,
     void *coef = nullptr;
     int *d_active = nullptr, *d_list = nullptr, *d_jl = nullptr, *d_nact = nullptr, *d_ids = nullptr;
     double *d_prev = nullptr;
-    unsigned long long *d_clock = nullptr;    // [0] launch start (globaltimer), [1] abort flag
+    unsigned long long *d_clock = nullptr;    // [0] launch start (globaltimer), [1] abort flag, [2] queue head
     auto release = [&]() {
         cudaFree(d_l4); cudaFree(buf[0]); cudaFree(buf[1]); cudaFree(coef);
         cudaFree(d_active); cudaFree(d_list); cudaFree(d_jl); cudaFree(d_nact); cudaFree(d_prev);
@@ -1490,8 +1599,8 @@ lbm_status lbm3d_local_keff_batch(const lbm3d_params *p, const float *kappa_dev,
     L3_CUDA2(cudaMemcpyAsync(d_l4, l4.data(), sizeof(int4) * n_leaves, cudaMemcpyHostToDevice, st));
     L3_CUDA2(cudaMalloc(&d_nact, sizeof(int)));
     L3_CUDA2(cudaMalloc(&d_ids, sizeof(int) * n_leaves));
-    L3_CUDA2(cudaMalloc(&d_clock, 2 * sizeof(unsigned long long)));
-    L3_CUDA2(cudaMemsetAsync(d_clock, 0, 2 * sizeof(unsigned long long), st));
+    L3_CUDA2(cudaMalloc(&d_clock, 3 * sizeof(unsigned long long)));
+    L3_CUDA2(cudaMemsetAsync(d_clock, 0, 3 * sizeof(unsigned long long), st));
     int dev = 0, optin = 0;
     L3_CUDA2(cudaGetDevice(&dev));
     L3_CUDA2(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
@@ -1503,9 +1612,11 @@ lbm_status lbm3d_local_keff_batch(const lbm3d_params *p, const float *kappa_dev,
         const int sz = kv.first;
         const int64_t s3 = (int64_t)sz * sz * sz;
         if (cluster_ok) {
-            const lbm_status cs = run_cluster_size(p, kappa_dev, d_l4, kv.second, d_ids, sz, m, nu, g_const, tol_rel,
-                                                   max_steps, check_every, optin, d_clock, keff_dev, status_dev,
-                                                   steps_dev, st);
+            lbm_status cs = run_pair_size(p, kappa_dev, d_l4, kv.second, d_ids, sz, m, nu, g_const, tol_rel, max_steps,
+                                          check_every, optin, d_clock, keff_dev, status_dev, steps_dev, st);
+            if (cs == LBM_EINVAL)
+                cs = run_cluster_size(p, kappa_dev, d_l4, kv.second, d_ids, sz, m, nu, g_const, tol_rel, max_steps,
+                                      check_every, optin, d_clock, keff_dev, status_dev, steps_dev, st);
             // LBM_ETIMEOUT is in the leaves' status already; LBM_EINVAL: the cube does not fit, take the global path
             if (cs == LBM_OK || cs == LBM_ETIMEOUT) continue;
             if (cs != LBM_EINVAL) {

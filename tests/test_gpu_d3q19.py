@@ -327,3 +327,20 @@ def test_d3q19_checkpoint_restart_is_bitwise(storage):
         with pytest.raises(lbm.LbmError) as ei:
             c.load_state(st[:-16])
         assert ei.value.status == lbm.LBM_EINVAL
+
+
+@pytest.mark.parametrize("sides,tau,steps,k", [(range(1, 10), 1.0, 130, 64), (range(10, 19), 0.8, 77, 10)])
+def test_local_keff3_two_jobs_a_cluster_match_oracle(sides, tau, steps, k):
+    """FP32 cubes of up to 18 cells run two jobs to a cluster of one to six CTAs; every side (odd ones leave
+    the last slab short) and a batch whose jobs are refilled more than once. 1e-5 is the FP32 bound above."""
+    kap = _field(40, 40, 40, seed=79)
+    kap[5, 6, 7] = 0.0
+    leaves = [((3 * s) % (41 - s), (5 * s) % (41 - s), (7 * s) % (41 - s), s) for s in sides]
+    leaves += [(x, y, z, 4) for z in range(0, 40, 4) for y in range(0, 40, 4) for x in range(0, 40, 4)] if 4 in sides else []
+    ke, st, n, _ = gpu_keff3(kap, leaves, tau, 0.1, 0.9, 1e-6, 0.0, steps, k=k)
+    assert (n == steps).all() and (st == 0).all()
+    for i in range(min(len(leaves), 40)):
+        x0, y0, z0, s = leaves[i]
+        cube = kap[z0:z0 + s, y0:y0 + s, x0:x0 + s].astype(np.float64)
+        ref = oracle.local_keff3(cube, tau, 0.1, 0.9, 1e-6, tol=0.0, max_steps=steps, check_every=k)["keff"]
+        np.testing.assert_allclose(ke[i], ref, rtol=0, atol=1e-5 * np.abs(np.diag(ref)).max())
