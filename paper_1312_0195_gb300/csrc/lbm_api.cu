@@ -2,6 +2,7 @@
 // CUDA-graph replay of the fused step, residual checks and field read-back.
 #include "lbm_internal.h"
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdarg>
@@ -110,6 +111,8 @@ int sm_count(int dev)
 
 using namespace lbm;
 
+constexpr int TILE_CHUNK = 4096;     // steps of one launch of the tile kernel at most
+
 struct lbm_grid {
     lbm_params p;
     double nu = 0, S = 1;
@@ -131,6 +134,12 @@ struct lbm_grid {
     int64_t t = 0;
     int sms = 1;
     bool fused = false;              // several steps per pass (multistep.cu) where a call takes several
+    TileGeom tiles{0, 0, 0, 0, 0};   // ntx > 0: a small lattice, stepped in shared memory (tiles.cu)
+    void *work = nullptr;            // holds partials, result, flags, tile_exch and tile_result
+    void *tile_exch = nullptr;       // exchanges between its CTAs
+    unsigned tile_base = 0;          // exchanges so far, and more
+    unsigned *tile_result = nullptr; // the checks' maxima of one launch, behind the exchanges
+    int *tile_err = nullptr;         // pinned, in h_result: a wait between its CTAs gave up
     struct Graph {
         cudaGraphExec_t exec;
         int kernels;                 // launches it holds
@@ -223,6 +232,48 @@ static cudaError_t enqueue_multi(const lbm_grid *g, int src_idx, int nlev, cudaS
     }
     auto a = make_args<float, float>(g, src, dst);
     return launch_multistep(LBM_F32, g->coef_mode, g->has_g, walls, &a, nlev, g->sms, st);
+}
+
+// n steps in one launch, the lattice resident in shared memory (tiles.cu), with the checks that fall into them
+// (check_every > 0); *checks: how many. Leaves the newest state in buf[cur]. The last check's maxima come back in
+// h_result as floats' bits.
+static cudaError_t enqueue_tiles(lbm_grid *g, int n, int check_every, int *checks)
+{
+    TileRun run{n, 0, check_every, g->tile_result, g->tile_exch, g->tile_base, g->tile_err};
+    *checks = 0;
+    if (check_every > 0) {
+        run.first_check = (int)(check_every - g->t % check_every);
+        *checks = n >= run.first_check ? 1 + (n - run.first_check) / check_every : 0;
+        if (*checks == 0) run.check_every = 0;
+    }
+    cudaError_t e = cudaSuccess;
+    if (*checks > 0) e = cudaMemsetAsync(g->tile_result, 0, 2 * sizeof(unsigned) * *checks, g->stream);
+    if (e != cudaSuccess) return e;
+    const void *src = g->buf[g->cur];
+    void *dst = g->buf[1 - g->cur];
+    const bool walls = g->p.bc == LBM_BC_WALLS_Y;
+    if (g->p.storage == LBM_F16) {
+        auto a = make_args<__half, float>(g, src, dst);
+        e = launch_tiles(LBM_F16, g->coef_mode, g->has_g, walls, &a, g->tiles, run, g->stream);
+    } else {
+        auto a = make_args<float, float>(g, src, dst);
+        e = launch_tiles(LBM_F32, g->coef_mode, g->has_g, walls, &a, g->tiles, run, g->stream);
+    }
+    if (e == cudaSuccess && *checks > 0)
+        e = cudaMemcpyAsync(g->h_result + 4, g->tile_result + 2 * (*checks - 1), 2 * sizeof(unsigned),
+                            cudaMemcpyDeviceToHost, g->stream);
+    if (e != cudaSuccess) return e;
+    g->tile_base += n / TILE_HALO + 1;
+    g->cur = 1 - g->cur;
+    return e;
+}
+
+static double tile_residual(const lbm_grid *g)
+{
+    float m[2];
+    std::memcpy(m, g->h_result + 4, sizeof m);
+    const double dmax = m[0], umax = m[1];
+    return umax > 0.0 ? dmax / umax : dmax;
 }
 
 // Graph of n steps starting from buf[parity], optionally followed by the residual pass (moments of
@@ -389,9 +440,7 @@ static void free_grid(lbm_grid *g)
     cudaFree(g->buf[1]);
     cudaFree(g->coef);
     cudaFree(g->gfield);
-    cudaFree(g->partials);
-    cudaFree(g->result);
-    cudaFree(g->flags);
+    cudaFree(g->work);
     if (g->h_result) cudaFreeHost(g->h_result);
     if (g->cap) cudaStreamDestroy(g->cap);
     cudaGetLastError();
@@ -477,10 +526,27 @@ lbm_status grid_create_impl(const lbm_params *p, const float *kappa_dev, const d
     LBM_GRID_CUDA(cudaMalloc(&g->buf[1], 9 * g->plane * sb));
     LBM_GRID_CUDA(cudaMalloc(&g->coef, ncoef * g->plane * cb));
     if (g->has_g) LBM_GRID_CUDA(cudaMalloc(&g->gfield, 2 * g->plane * cb));
-    LBM_GRID_CUDA(cudaMalloc(&g->partials, 4 * sizeof(double) * g->L.mom_blocks));
-    LBM_GRID_CUDA(cudaMalloc(&g->result, 4 * sizeof(double)));
-    LBM_GRID_CUDA(cudaMalloc(&g->flags, 2 * sizeof(unsigned)));
     LBM_GRID_CUDA(cudaMallocHost(&g->h_result, 8 * sizeof(double)));
+    g->tile_err = reinterpret_cast<int *>(g->h_result + 6);
+    *g->tile_err = 0;
+    if (g->fused) g->tiles = tile_geometry(p->storage, g->coef_mode, g->has_g, p->nx, p->ny, sms);
+    // one allocation for the reductions' small arrays and the exchanges of the tile kernel; no room for the
+    // latter: stepped in passes over memory
+    const size_t small = 4 * sizeof(double) * (g->L.mom_blocks + 1) + 4 * sizeof(unsigned);     // a multiple of 16
+    const size_t exch = g->tiles.ntx > 0 ? tile_exchange_bytes(n) : 0;
+    if (g->tiles.ntx > 0 &&
+        cudaMalloc(&g->work, small + exch + 2 * sizeof(unsigned) * TILE_CHUNK) != cudaSuccess) {
+        cudaGetLastError();
+        g->work = nullptr;
+        g->tiles.ntx = 0;
+    }
+    if (g->tiles.ntx == 0) LBM_GRID_CUDA(cudaMalloc(&g->work, small));
+    g->partials = static_cast<double *>(g->work);
+    g->result = g->partials + 4 * g->L.mom_blocks;
+    g->flags = reinterpret_cast<unsigned *>(g->result + 4);
+    g->tile_exch = reinterpret_cast<char *>(g->work) + small;
+    g->tile_result = reinterpret_cast<unsigned *>(static_cast<char *>(g->tile_exch) + exch);
+    if (g->tiles.ntx > 0) LBM_GRID_CUDA(cudaMemsetAsync(g->tile_exch, 0, exch, g->stream));
 
     cudaStream_t st = g->stream;
     // rest state: deviations are zero in both buffers (state of step -1 and -2)
@@ -577,8 +643,36 @@ lbm_status lbm_step(lbm_grid *g, int64_t max_steps, double tol_rel, int32_t chec
     const int CHUNK = 1024;
     int64_t left = max_steps, done = 0;
     double resid = -1.0;
-    bool converged = false, checked = false;
+    bool converged = false, checked = false, in_tiles = false;      // in_tiles: where the last check ran
     while (left > 0) {
+        // one launch of the tile kernel runs up to the next value the host needs
+        int64_t m = left < TILE_CHUNK ? left : TILE_CHUNK;
+        if (tol_rel > 0.0) m = std::min<int64_t>(m, check_every - g->t % check_every);
+        if (g->tiles.ntx > 0 && m >= TILES_FROM) {
+            int checks = 0;
+            const cudaError_t e = enqueue_tiles(g, (int)m, check_every, &checks);
+            if (e == cudaErrorCooperativeLaunchTooLarge) {       // a stream with a part of the SMs
+                cudaGetLastError();
+                g->tiles.ntx = 0;
+                continue;
+            }
+            LBM_CUDA(e);
+            count_launches(1);
+            g->t += m;
+            done += m;
+            left -= m;
+            if (checks == 0) continue;
+            checked = in_tiles = true;
+            if (tol_rel > 0.0) {
+                LBM_CUDA(cudaStreamSynchronize(g->stream));
+                resid = tile_residual(g);
+                if (resid <= tol_rel) {
+                    converged = true;
+                    break;
+                }
+            }
+            continue;
+        }
         int64_t n = left < CHUNK ? left : CHUNK;
         int check = 0;
         if (check_every > 0) {
@@ -599,6 +693,7 @@ lbm_status lbm_step(lbm_grid *g, int64_t max_steps, double tol_rel, int32_t chec
         g->cur = gr.cur;
         if (check) {
             checked = true;
+            in_tiles = false;
             if (tol_rel > 0.0) {      // the stop test needs the value now; otherwise read it at the end
                 LBM_CUDA(cudaStreamSynchronize(g->stream));
                 const double dmax = g->h_result[0], umax = g->h_result[1];
@@ -611,7 +706,13 @@ lbm_status lbm_step(lbm_grid *g, int64_t max_steps, double tol_rel, int32_t chec
         }
     }
     LBM_CUDA(cudaStreamSynchronize(g->stream));
-    if (checked && tol_rel <= 0.0) {
+    if (*(volatile int *)g->tile_err) {                      // the state is not valid any more
+        *g->tile_err = 0;
+        return fail(LBM_ECUDA, "a wait between the tiles of the lattice gave up");
+    }
+    if (checked && tol_rel <= 0.0 && in_tiles) {
+        resid = tile_residual(g);
+    } else if (checked && tol_rel <= 0.0) {
         const double dmax = g->h_result[0], umax = g->h_result[1];
         resid = umax > 0.0 ? dmax / umax : dmax;
     }

@@ -83,6 +83,34 @@ bool multistep_ok(int storage, int coef_mode, int nx, int ny, int guo);
 cudaError_t launch_multistep(int storage, int coef_mode, bool gfield, bool walls, const void *args, int nlev, int sms,
                              cudaStream_t st);
 
+// ---- many steps per launch on small lattices (tiles.cu) ---------------------------
+constexpr int TILE_HALO = 4;            // steps between two exchanges, and cells of halo
+struct TileGeom {
+    int ntx, nty;     // tiles along x and y (0: the lattice does not fit)
+    int W, H;         // cells of the largest tile with its halo
+    int ctas;         // CTAs, two tiles each
+};
+TileGeom tile_geometry(int storage, int coef_mode, bool gfield, int nx, int ny, int sms);
+// Steps of a launch at least (more than TILE_HALO: an exchange has to take place). Filling shared memory and writing
+// it back costs 15 to 20 us: a call of 8 steps took 23 us at 128 x 64 and 39 us at 500 x 500, in passes of four 25 and
+// 32 us; one of 12 steps 27 and 48 us against 33 and 43 us, one of 24 steps 38 and 73 us against 48 and 75 us.
+constexpr int TILES_FROM = 12;
+constexpr size_t tile_exchange_bytes(int64_t cells) { return (size_t)cells * 2 * 3 * 16; }
+// One launch: `steps` steps from the state in src, with the residual's maxima (bits of max |du| and max |u|) after
+// step first_check and every check_every-th step on (check_every = 0: none) raised in result[2 c], result[2 c + 1] for
+// the c-th of them (zeroed before). dst gets the newest state, src the one before it. exch: the exchanges' words,
+// tile_exchange_bytes, zeroed once; base: the number of exchanges that have gone through it; err: set if a wait
+// between CTAs gave up.
+struct TileRun {
+    int steps, first_check, check_every;
+    unsigned *result;
+    void *exch;
+    unsigned base;
+    int *err;
+};
+cudaError_t launch_tiles(int storage, int coef_mode, bool gfield, bool walls, const void *args, const TileGeom &g,
+                         const TileRun &run, cudaStream_t st);
+
 // ---- launch counter (lbm_api.cu) ----------------------------------------------
 void count_launches(int64_t n);
 

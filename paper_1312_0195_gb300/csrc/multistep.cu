@@ -25,7 +25,7 @@
 // (0.30 ms a pass). Warps of one SM take neighbouring strips, which saves 7 % of the time (L1 hits on the
 // sectors that two strips share).
 #include "lbm_internal.h"
-#include "pair_ops.cuh"
+#include "pair_step.cuh"
 
 #include <type_traits>
 
@@ -82,13 +82,6 @@ __device__ __forceinline__ typename PairT<T>::V load_pair(const T *plane, unsign
     }
 }
 
-// Drag coefficients and force of a pair.
-template <int COEF, bool GF>
-struct PairCoef {
-    float2 c0, c1, c2, c3, gx, gy;
-};
-template <int COEF, bool GF> constexpr int ncoef() { return (COEF == COEF_TENSOR ? 4 : 1) + (GF ? 2 : 0); }
-
 // Rows are copied into shared memory AHEAD positions before they are used, each lane its own pairs, so a lane
 // waits only for its own copies and no barrier is needed. A slot is overwritten one position after its
 // values were last read.
@@ -114,54 +107,6 @@ __device__ __forceinline__ void stage_pair(typename PairT<T>::V *dst, const T *p
         copy_async<E>(&dst->x, at(plane, (row + x0) * E));
         copy_async<E>(&dst->y, at(plane, (row + x1) * E));
     }
-}
-
-// The collision of two cells given their streamed deviations: collide_cell of step.cu (simplified
-// scheme), with the products and sums that the compiler fuses there fused here explicitly.
-template <int COEF, bool GF>
-__device__ __forceinline__ void collide_pair(float2 (&g)[Q], const PairCoef<COEF, GF> &k, float rho0, float half_eps,
-                                             float omega, float two_tau, float omt)
-{
-    float2 drho = g[0];
-#pragma unroll
-    for (int a = 1; a < Q; ++a) drho = add2(drho, g[a]);
-    float2 mx = sub2(g[1], g[3]);
-    mx = add2(mx, g[5]);
-    mx = sub2(mx, g[6]);
-    mx = sub2(mx, g[7]);
-    mx = add2(mx, g[8]);
-    float2 my = sub2(g[2], g[4]);
-    my = add2(my, g[5]);
-    my = add2(my, g[6]);
-    my = sub2(my, g[7]);
-    my = sub2(my, g[8]);
-    const float2 rho = add2(dup2(rho0), drho);
-    const float2 h = mul2(dup2(half_eps), rho);
-    const float2 rx = fma2(h, k.gx, mx), ry = fma2(h, k.gy, my);
-    float2 rux, ruy;
-    if constexpr (COEF == COEF_SCALAR) {
-        const float2 m = make_float2(-k.c0.x, -k.c0.y);
-        rux = fma2(m, rx, rx);
-        ruy = fma2(m, ry, ry);
-    } else {
-        rux = sub2(rx, fma2(k.c0, rx, mul2(k.c1, ry)));
-        ruy = sub2(ry, fma2(k.c2, rx, mul2(k.c3, ry)));
-    }
-    const float2 ux = fma2(dup2(omt), mx, mul2(dup2(two_tau), rux));
-    const float2 uy = fma2(dup2(omt), my, mul2(dup2(two_tau), ruy));
-    const float2 sp = add2(ux, uy), sm = sub2(ux, uy);
-    const float w0 = float(4.0 / 9.0), w1 = float(1.0 / 9.0), w2 = float(1.0 / 36.0);
-    // g + omega (w q - g): the inner difference is kept with its sign turned, -(w q - g)
-    auto relax = [&](float2 &p, float w, float2 q) { p = fma2(dup2(-omega), fma2(dup2(-w), q, p), p); };
-    relax(g[0], w0, drho);
-    relax(g[1], w1, fma2(dup2(3.0f), ux, drho));
-    relax(g[3], w1, fma2(dup2(-3.0f), ux, drho));
-    relax(g[2], w1, fma2(dup2(3.0f), uy, drho));
-    relax(g[4], w1, fma2(dup2(-3.0f), uy, drho));
-    relax(g[5], w2, fma2(dup2(3.0f), sp, drho));
-    relax(g[7], w2, fma2(dup2(-3.0f), sp, drho));
-    relax(g[8], w2, fma2(dup2(3.0f), sm, drho));
-    relax(g[6], w2, fma2(dup2(-3.0f), sm, drho));
 }
 
 // Rows on their way from one step to the next: populations with e_y = 0 (0, 1, 3) wait one row, those
@@ -423,8 +368,9 @@ cudaError_t launch_c(bool gf, bool walls, const StepArgs<T, float> &a, int nlev,
 }  // namespace
 
 // Guo's scheme and FP16 with a tensor K* keep the one-step kernel; so do lattices too small for the
-// single wrap of a row index. Elsewhere a fused pass was faster at every size measured (128 x 64:
-// 2.4 us a step against 3.3; 517 x 389, odd rows: 3.3 against 4.3; 4096 x 4096: 53 against 196).
+// single wrap of a row index. Elsewhere a fused pass was faster at every size measured (us a step; 128 x 64:
+// 2.0 against 2.6; 517 x 389, odd rows: 2.9 against 4.0; 4096 x 4096: 53 against 196). Long runs of small
+// lattices go on to tiles.cu.
 bool multistep_ok(int storage, int coef_mode, int nx, int ny, int guo)
 {
     if ((int64_t)nx * ny >= (int64_t)1 << 30) return false;      // 32-bit byte offsets within a plane

@@ -402,3 +402,36 @@ def test_fused_passes_equal_single_steps_bitwise(storage, nx, ny, monkeypatch):
                     got.append((resid, st.cpu().numpy()))
             assert got[0][0] == got[1][0]
             np.testing.assert_array_equal(got[0][1], got[1][1])
+
+
+@pytest.mark.parametrize("storage", [0, 1])
+@pytest.mark.parametrize("nx,ny", [(8, 8), (9, 16), (17, 8), (257, 255), (517, 389), (500, 540)])
+def test_resident_tiles_equal_single_steps_bitwise(storage, nx, ny, monkeypatch):
+    """Small lattices are stepped in shared memory, residual checks included; the arithmetic is that of the
+    one-step kernel, so both states, every residual and the step at which a run stops agree bit for bit.
+    Sizes: one tile, unequal tiles, the largest lattice; steps and checks at and beside an exchange (every
+    four steps) and below the shortest run that takes this way."""
+    import torch
+    lbm = _lbm()
+    kap = torch.from_numpy(synth.lognormal_kappa(nx, ny, 4.0, 1.5, seed=nx + ny).astype(np.float32)).cuda()
+    field = torch.rand((2, ny, nx), generator=torch.Generator().manual_seed(3)).cuda() * 1e-6
+    for walls in (False, True):
+        got = []
+        for single in (False, True):
+            if single:
+                monkeypatch.setenv("LBM_STEP_VEC", "1")
+            else:
+                monkeypatch.delenv("LBM_STEP_VEC", raising=False)
+            p = lbm.Params(nx=nx, ny=ny, tau=0.7, gx=1e-6, gy=3e-7, storage=storage,
+                           bc=lbm.LBM_BC_WALLS_Y if walls else lbm.LBM_BC_PERIODIC)
+            with lbm.Grid(p, kap, field if walls else None) as G:
+                out = []
+                for n, check in ((11, 0), (12, 12), (13, 1), (16, 3), (17, 17), (35, 4)):
+                    out.append(G.step(n, 0.0, check)[1])
+                    st = torch.empty(lbm.lbm_grid_state_bytes(G.handle), dtype=torch.uint8, device="cuda")
+                    lbm.lbm_grid_save_state(G.handle, st)
+                    out.append(st.cpu().numpy())
+                out.append(G.step(400, 0.02, 13)[:2])
+                got.append(out)
+        for a, b in zip(*got):
+            np.testing.assert_array_equal(a, b)
