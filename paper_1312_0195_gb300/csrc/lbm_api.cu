@@ -135,7 +135,8 @@ struct lbm_grid {
     int sms = 1;
     bool fused = false;              // several steps per pass (multistep.cu) where a call takes several
     TileGeom tiles{0, 0, 0, 0, 0};   // ntx > 0: a small lattice, stepped in shared memory (tiles.cu)
-    void *work = nullptr;            // holds partials, result, flags, tile_exch and tile_result
+    unsigned *check_bits = nullptr;  // a check's maxima inside a pass
+    void *work = nullptr;            // holds partials, result, flags, check_bits, tile_exch and tile_result
     void *tile_exch = nullptr;       // exchanges between its CTAs
     unsigned tile_base = 0;          // exchanges so far, and more
     unsigned *tile_result = nullptr; // the checks' maxima of one launch, behind the exchanges
@@ -220,18 +221,18 @@ static cudaError_t enqueue_moments(const lbm_grid *g, int cur_idx, int prev_idx,
     }
 }
 
-// nlev steps in one pass over memory (multistep.cu).
-static cudaError_t enqueue_multi(const lbm_grid *g, int src_idx, int nlev, cudaStream_t st)
+// nlev steps in one pass over memory (multistep.cu); check: with the residual's maxima after the last but one.
+static cudaError_t enqueue_multi(const lbm_grid *g, int src_idx, int nlev, unsigned *check, cudaStream_t st)
 {
     const void *src = g->buf[src_idx];
     void *dst = g->buf[1 - src_idx];
     const bool walls = g->p.bc == LBM_BC_WALLS_Y;
     if (g->p.storage == LBM_F16) {
         auto a = make_args<__half, float>(g, src, dst);
-        return launch_multistep(LBM_F16, g->coef_mode, g->has_g, walls, &a, nlev, g->sms, st);
+        return launch_multistep(LBM_F16, g->coef_mode, g->has_g, walls, &a, nlev, g->sms, check, st);
     }
     auto a = make_args<float, float>(g, src, dst);
-    return launch_multistep(LBM_F32, g->coef_mode, g->has_g, walls, &a, nlev, g->sms, st);
+    return launch_multistep(LBM_F32, g->coef_mode, g->has_g, walls, &a, nlev, g->sms, check, st);
 }
 
 // n steps in one launch, the lattice resident in shared memory (tiles.cu), with the checks that fall into them
@@ -268,7 +269,8 @@ static cudaError_t enqueue_tiles(lbm_grid *g, int n, int check_every, int *check
     return e;
 }
 
-static double tile_residual(const lbm_grid *g)
+// The residual of a check that left its maxima as floats' bits.
+static double bits_residual(const lbm_grid *g)
 {
     float m[2];
     std::memcpy(m, g->h_result + 4, sizeof m);
@@ -279,7 +281,11 @@ static double tile_residual(const lbm_grid *g)
 // Graph of n steps starting from buf[parity], optionally followed by the residual pass (moments of
 // the last two states, reduction, copy to pinned host). Where the grid fuses steps, the passes take
 // MULTISTEP_MAX steps each; with `pair` the last step is one of its own, so that the two
-// buffers end up holding the last two states (the residual and a checkpoint read both).
+// buffers end up holding the last two states (the residual and a checkpoint read both). check = CHECK_INSIDE: the
+// residual after step n - 1 comes from the last pass, of MULTISTEP_MAX steps, which has both states' velocities at
+// hand: 4096 x 4096 with a check every 64 steps then takes 16 equal passes, where a shorter pass, a single
+// step and the residual pass used to take the place of the last.
+constexpr int CHECK_INSIDE = 2;
 static lbm_status get_graph(lbm_grid *g, int n, int parity, int check, int pair, lbm_grid::Graph *out)
 {
     if (!g->fused) pair = 0;
@@ -293,17 +299,22 @@ static lbm_status get_graph(lbm_grid *g, int n, int parity, int check, int pair,
     LBM_CUDA(cudaStreamBeginCapture(g->cap, cudaStreamCaptureModeThreadLocal));
     cudaError_t err = cudaSuccess;
     int idx = parity, kernels = 0;
+    const bool inside = check == CHECK_INSIDE;
+    if (inside) err = cudaMemsetAsync(g->check_bits, 0, 2 * sizeof(unsigned), g->cap);
     for (int left = n; left > 0 && err == cudaSuccess; ++kernels) {
         int take = 1;
+        const bool last = inside && left == MULTISTEP_MAX;
         if (g->fused) {
-            take = left - (pair || check ? 1 : 0);
+            take = inside && !last ? left - MULTISTEP_MAX : left - (pair || check == 1 ? 1 : 0);
             take = take < 1 ? 1 : (take > MULTISTEP_MAX ? MULTISTEP_MAX : take);
         }
-        err = take > 1 ? enqueue_multi(g, idx, take, g->cap) : enqueue_step(g, idx, g->cap);
+        err = take > 1 ? enqueue_multi(g, idx, take, last ? g->check_bits : nullptr, g->cap) : enqueue_step(g, idx, g->cap);
         idx = 1 - idx;
         left -= take;
     }
-    if (check && err == cudaSuccess) {
+    if (inside && err == cudaSuccess)
+        err = cudaMemcpyAsync(g->h_result + 4, g->check_bits, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, g->cap);
+    if (check == 1 && err == cudaSuccess) {
         err = enqueue_moments(g, idx, 1 - idx, nullptr, nullptr, nullptr, g->cap);
         if (err == cudaSuccess) err = launch_reduce_partials(g->partials, g->L.mom_blocks, g->result, g->cap);
         if (err == cudaSuccess)
@@ -544,6 +555,7 @@ lbm_status grid_create_impl(const lbm_params *p, const float *kappa_dev, const d
     g->partials = static_cast<double *>(g->work);
     g->result = g->partials + 4 * g->L.mom_blocks;
     g->flags = reinterpret_cast<unsigned *>(g->result + 4);
+    g->check_bits = g->flags + 2;
     g->tile_exch = reinterpret_cast<char *>(g->work) + small;
     g->tile_result = reinterpret_cast<unsigned *>(static_cast<char *>(g->tile_exch) + exch);
     if (g->tiles.ntx > 0) LBM_GRID_CUDA(cudaMemsetAsync(g->tile_exch, 0, exch, g->stream));
@@ -643,7 +655,7 @@ lbm_status lbm_step(lbm_grid *g, int64_t max_steps, double tol_rel, int32_t chec
     const int CHUNK = 1024;
     int64_t left = max_steps, done = 0;
     double resid = -1.0;
-    bool converged = false, checked = false, in_tiles = false;      // in_tiles: where the last check ran
+    bool converged = false, checked = false, as_bits = false;       // as_bits: how the last check left its result
     while (left > 0) {
         // one launch of the tile kernel runs up to the next value the host needs
         int64_t m = left < TILE_CHUNK ? left : TILE_CHUNK;
@@ -662,10 +674,10 @@ lbm_status lbm_step(lbm_grid *g, int64_t max_steps, double tol_rel, int32_t chec
             done += m;
             left -= m;
             if (checks == 0) continue;
-            checked = in_tiles = true;
+            checked = as_bits = true;
             if (tol_rel > 0.0) {
                 LBM_CUDA(cudaStreamSynchronize(g->stream));
-                resid = tile_residual(g);
+                resid = bits_residual(g);
                 if (resid <= tol_rel) {
                     converged = true;
                     break;
@@ -677,7 +689,10 @@ lbm_status lbm_step(lbm_grid *g, int64_t max_steps, double tol_rel, int32_t chec
         int check = 0;
         if (check_every > 0) {
             const int64_t to_next = check_every - (g->t % check_every);
-            if (to_next <= n) {
+            if (g->fused && tol_rel <= 0.0 && to_next + 1 >= MULTISTEP_MAX && to_next < n && to_next + 1 < left) {
+                n = to_next + 1;
+                check = CHECK_INSIDE;
+            } else if (to_next <= n) {
                 n = to_next;
                 check = 1;
             }
@@ -693,7 +708,7 @@ lbm_status lbm_step(lbm_grid *g, int64_t max_steps, double tol_rel, int32_t chec
         g->cur = gr.cur;
         if (check) {
             checked = true;
-            in_tiles = false;
+            as_bits = check == CHECK_INSIDE;
             if (tol_rel > 0.0) {      // the stop test needs the value now; otherwise read it at the end
                 LBM_CUDA(cudaStreamSynchronize(g->stream));
                 const double dmax = g->h_result[0], umax = g->h_result[1];
@@ -710,8 +725,8 @@ lbm_status lbm_step(lbm_grid *g, int64_t max_steps, double tol_rel, int32_t chec
         *g->tile_err = 0;
         return fail(LBM_ECUDA, "a wait between the tiles of the lattice gave up");
     }
-    if (checked && tol_rel <= 0.0 && in_tiles) {
-        resid = tile_residual(g);
+    if (checked && tol_rel <= 0.0 && as_bits) {
+        resid = bits_residual(g);
     } else if (checked && tol_rel <= 0.0) {
         const double dmax = g->h_result[0], umax = g->h_result[1];
         resid = umax > 0.0 ? dmax / umax : dmax;

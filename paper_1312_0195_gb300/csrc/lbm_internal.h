@@ -81,7 +81,7 @@ constexpr int MULTISTEP_MIN_ROWS = 4;   // rows of a warp's segment at least: fe
                                         // they gain in parallel warps (256 x 256: 2.9 us a step at 4, 3.3 at 2)
 bool multistep_ok(int storage, int coef_mode, int nx, int ny, int guo);
 cudaError_t launch_multistep(int storage, int coef_mode, bool gfield, bool walls, const void *args, int nlev, int sms,
-                             cudaStream_t st);
+                             unsigned *check, cudaStream_t st);
 
 // ---- many steps per launch on small lattices (tiles.cu) ---------------------------
 constexpr int TILE_HALO = 4;            // steps between two exchanges, and cells of halo

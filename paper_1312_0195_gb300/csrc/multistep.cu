@@ -122,6 +122,7 @@ struct MultiGeom {
     int strips;      // column strips
     int segs;        // row segments
     int seg_rows;    // rows of a segment
+    unsigned *check; // CHECK: bits of max |du|, max |u|
 };
 
 // Warps per SM: the rows in flight and a collision take up to 168 registers in FP32, 128 in FP16.
@@ -134,7 +135,12 @@ constexpr size_t warp_smem()
     return (size_t)RING * Q * 32 * 2 * sizeof(T) + (size_t)CRING * ncoef<COEF, GF>() * 32 * sizeof(float2);
 }
 
-template <typename T, int COEF, bool GF, bool WALLS, bool ALIGNED>
+// CHECK (with LEV steps): also raises *m.check to the maxima of the residual after the pass's third step. The third
+// and fourth step pull the two states it compares, so their velocities are at hand; the fourth's row is one
+// behind, for which the third's velocity waits one position.
+// It takes the place of a shorter pass, a single step and a pass of the residual kernel: 4096 x 4096, 256 steps with a
+// check every 64, 15.6 -> 14.6 ms (FP16 15.4 -> 14.7); the check alone costs its pass the divisions.
+template <typename T, int COEF, bool GF, bool WALLS, bool ALIGNED, bool CHECK>
 __global__ void __launch_bounds__(ms_warps<T>() * 32, 1) multi_step_kernel(StepArgs<T, float> a, MultiGeom m)
 {
     using V = typename PairT<T>::V;
@@ -204,8 +210,12 @@ __global__ void __launch_bounds__(ms_warps<T>() * 32, 1) multi_step_kernel(StepA
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    // one step of row r, the warp's j-th row: p holds its sources before the one-column shift
-    auto step_row = [&](int r, int j, V (&p)[Q]) {
+    float2 pu[2], pv[2];                             // velocity at the third step, by parity of the position
+    float dmax = 0.0f, umax = 0.0f;
+    if constexpr (CHECK) pu[0] = pu[1] = pv[0] = pv[1] = dup2(0.0f);
+    // step `lev` of row r, the warp's j-th row, at a position of parity P: p holds its sources before the one-column
+    // shift
+    auto step_row = [&](int lev, int P, int r, int j, V (&p)[Q]) {
         const float2 *c = coefs + ((unsigned)j % CRING) * (NC * 32);
         PairCoef<COEF, GF> k;
         k.c0 = c[0];
@@ -228,6 +238,27 @@ __global__ void __launch_bounds__(ms_warps<T>() * 32, 1) multi_step_kernel(StepA
         g[6] = to_f2(lo ? p[6] : r6);
         g[7] = to_f2(hi ? p[7] : r7);
         g[8] = to_f2(hi ? p[8] : l8);
+        if constexpr (CHECK) {
+            if (lev >= LEV - 2) {
+                const Flow2 f = flow_pair<COEF, GF>(g, k, a.rho0, a.half_eps);
+                const float2 u = make_float2(f.rux.x / f.rho.x, f.rux.y / f.rho.y);
+                const float2 v = make_float2(f.ruy.x / f.rho.x, f.ruy.y / f.rho.y);
+                if (lev == LEV - 2) {
+                    pu[P] = u;
+                    pv[P] = v;
+                } else if (r >= ya && r < yb) {
+                    const float2 du = sub2(u, pu[1 - P]), dv = sub2(v, pv[1 - P]);
+                    if (st0) {
+                        dmax = fmaxf(dmax, fmaxf(fabsf(du.x), fabsf(dv.x)));
+                        umax = fmaxf(umax, fmaxf(fabsf(u.x), fabsf(v.x)));
+                    }
+                    if (st1) {
+                        dmax = fmaxf(dmax, fmaxf(fabsf(du.y), fabsf(dv.y)));
+                        umax = fmaxf(umax, fmaxf(fabsf(u.y), fabsf(v.y)));
+                    }
+                }
+            }
+        }
         collide_pair<COEF, GF>(g, k, a.rho0, a.half_eps, a.omega, a.two_tau, a.one_m_two_tau);
 #pragma unroll
         for (int q = 0; q < Q; ++q) p[q] = from_f2<V>(g[q]);
@@ -240,7 +271,7 @@ __global__ void __launch_bounds__(ms_warps<T>() * 32, 1) multi_step_kernel(StepA
         for (int j = 0; j < 3; ++j)
             line[k].up[0][j] = line[k].up[1][j] = line[k].mid[j] = line[k].down[j] = from_f2<V>(dup2(0.0f));
 
-    const int nlev = m.nlev;
+    const int nlev = CHECK ? LEV : m.nlev;
     const int i0 = ya - (nlev - 1), n = yb - ya + 2 * (nlev - 1);
 #pragma unroll
     for (int j = 0; j < AHEAD; ++j) stage_row(i0 + j, j);
@@ -260,7 +291,7 @@ __global__ void __launch_bounds__(ms_warps<T>() * 32, 1) multi_step_kernel(StepA
             load_next(i + 1);
         }
         stage_row(i + AHEAD, j + AHEAD);
-        step_row(i, j, p);
+        step_row(0, P, i, j, p);
         int r = i;                                   // the row p now holds
 #pragma unroll
         for (int k = 0; k < LEV - 1; ++k) {
@@ -291,7 +322,7 @@ __global__ void __launch_bounds__(ms_warps<T>() * 32, 1) multi_step_kernel(StepA
                 }
 #pragma unroll
                 for (int q = 0; q < Q; ++q) p[q] = s[q];
-                step_row(r, j - (k + 1), p);
+                step_row(k + 1, P, r, j - (k + 1), p);
             }
         }
         if (r >= ya && r < yb) {
@@ -317,20 +348,29 @@ __global__ void __launch_bounds__(ms_warps<T>() * 32, 1) multi_step_kernel(StepA
         march(j + 1, std::integral_constant<int, 1>{});
     }
     asm volatile("cp.async.wait_all;" ::: "memory");   // rows staged past the end
+    if constexpr (CHECK) {                             // the order of non-negative floats is that of their bits
+        const unsigned d = __reduce_max_sync(0xffffffffu, __float_as_uint(dmax));
+        const unsigned u = __reduce_max_sync(0xffffffffu, __float_as_uint(umax));
+        if (lane == 0) {
+            atomicMax(m.check, d);
+            atomicMax(m.check + 1, u);
+        }
+    }
 }
 
-template <typename T, int COEF, bool GF, bool WALLS, bool ALIGNED>
-cudaError_t launch_t(const StepArgs<T, float> &a, int nlev, int sms, cudaStream_t st)
+template <typename T, int COEF, bool GF, bool WALLS, bool ALIGNED, bool CHECK>
+cudaError_t launch_t(const StepArgs<T, float> &a, int nlev, int sms, unsigned *check, cudaStream_t st)
 {
     constexpr size_t per_warp = warp_smem<T, COEF, GF>();
     constexpr int by_smem = (int)(231424 / per_warp);            // 227 KB, 1 KB of it reserved per CTA
     constexpr int sm_warps = by_smem < ms_warps<T>() ? by_smem : ms_warps<T>();
-    const auto kern = multi_step_kernel<T, COEF, GF, WALLS, ALIGNED>;
+    const auto kern = multi_step_kernel<T, COEF, GF, WALLS, ALIGNED, CHECK>;
     const cudaError_t e =
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(per_warp * sm_warps));
     if (e != cudaSuccess) return e;
     MultiGeom m;
     m.nlev = nlev;
+    m.check = check;
     m.strips = (a.nx + USEFUL - 1) / USEFUL;
     // one wave of resident warps; segments of at least MULTISTEP_MIN_ROWS rows
     int segs = sms * sm_warps / m.strips;
@@ -348,11 +388,13 @@ cudaError_t launch_t(const StepArgs<T, float> &a, int nlev, int sms, cudaStream_
 }
 
 template <typename T, int COEF>
-cudaError_t launch_c(bool gf, bool walls, const StepArgs<T, float> &a, int nlev, int sms, cudaStream_t st)
+cudaError_t launch_c(bool gf, bool walls, const StepArgs<T, float> &a, int nlev, int sms, unsigned *check, cudaStream_t st)
 {
     const bool al = a.nx % 2 == 0;
 #define LBM_MS_CASE(GFv, WLv, ALv)                       \
-    if (gf == GFv && walls == WLv && al == ALv) return launch_t<T, COEF, GFv, WLv, ALv>(a, nlev, sms, st);
+    if (gf == GFv && walls == WLv && al == ALv)          \
+        return check ? launch_t<T, COEF, GFv, WLv, ALv, true>(a, nlev, sms, check, st) \
+                     : launch_t<T, COEF, GFv, WLv, ALv, false>(a, nlev, sms, check, st);
     LBM_MS_CASE(false, false, false)
     LBM_MS_CASE(false, false, true)
     LBM_MS_CASE(false, true, false)
@@ -379,17 +421,17 @@ bool multistep_ok(int storage, int coef_mode, int nx, int ny, int guo)
 }
 
 cudaError_t launch_multistep(int storage, int coef_mode, bool gfield, bool walls, const void *args, int nlev, int sms,
-                             cudaStream_t st)
+                             unsigned *check, cudaStream_t st)
 {
-    if (nlev < 1 || nlev > LEV) return cudaErrorInvalidValue;
+    if (nlev < 1 || nlev > LEV || (check && nlev != LEV)) return cudaErrorInvalidValue;
     if (storage == LBM_F32) {
         const StepArgs<float, float> &a = *static_cast<const StepArgs<float, float> *>(args);
-        return coef_mode == COEF_SCALAR ? launch_c<float, COEF_SCALAR>(gfield, walls, a, nlev, sms, st)
-                                        : launch_c<float, COEF_TENSOR>(gfield, walls, a, nlev, sms, st);
+        return coef_mode == COEF_SCALAR ? launch_c<float, COEF_SCALAR>(gfield, walls, a, nlev, sms, check, st)
+                                        : launch_c<float, COEF_TENSOR>(gfield, walls, a, nlev, sms, check, st);
     }
     if (storage == LBM_F16 && coef_mode == COEF_SCALAR)
         return launch_c<__half, COEF_SCALAR>(gfield, walls, *static_cast<const StepArgs<__half, float> *>(args), nlev,
-                                             sms, st);
+                                             sms, check, st);
     return cudaErrorInvalidValue;
 }
 

@@ -435,3 +435,34 @@ def test_resident_tiles_equal_single_steps_bitwise(storage, nx, ny, monkeypatch)
                 got.append(out)
         for a, b in zip(*got):
             np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("storage", [0, 1])
+@pytest.mark.parametrize("nx,ny", [(1024, 520), (777, 401)])
+def test_checks_inside_fused_passes_equal_single_steps_bitwise(storage, nx, ny, monkeypatch):
+    """A check with at least one step after it is taken inside a pass of four steps, from the velocities that its
+    third and fourth step form. Residual and states agree bit for bit with single steps and the residual pass, at
+    even and odd columns, with walls and a force field, and for checks too close together for such a pass."""
+    import torch
+    lbm = _lbm()
+    kap = torch.from_numpy(synth.lognormal_kappa(nx, ny, 4.0, 1.5, seed=nx + ny).astype(np.float32)).cuda()
+    field = torch.rand((2, ny, nx), generator=torch.Generator().manual_seed(3)).cuda() * 1e-6
+    for walls in (False, True):
+        got = []
+        for single in (False, True):
+            if single:
+                monkeypatch.setenv("LBM_STEP_VEC", "1")
+            else:
+                monkeypatch.delenv("LBM_STEP_VEC", raising=False)
+            p = lbm.Params(nx=nx, ny=ny, tau=0.7, gx=1e-6, gy=3e-7, storage=storage,
+                           bc=lbm.LBM_BC_WALLS_Y if walls else lbm.LBM_BC_PERIODIC)
+            with lbm.Grid(p, kap, field if walls else None) as G:
+                out = []
+                for n, check in ((66, 64), (70, 64), (31, 5), (14, 3), (6, 4), (9, 1), (9, 2)):
+                    out.append(G.step(n, 0.0, check)[1])
+                    st = torch.empty(lbm.lbm_grid_state_bytes(G.handle), dtype=torch.uint8, device="cuda")
+                    lbm.lbm_grid_save_state(G.handle, st)
+                    out.append(st.cpu().numpy())
+                got.append(out)
+        for a, b in zip(*got):
+            np.testing.assert_array_equal(a, b)
