@@ -113,6 +113,15 @@ using namespace lbm;
 
 constexpr int TILE_CHUNK = 4096;     // steps of one launch of the tile kernel at most
 
+// What a call reads back, in one piece of device memory.
+struct Outcome {
+    double sums[4];        // of moments_kernel: max |du|, max |u|, sum u, sum v
+    unsigned flags[2];     // error bits of the coefficients, bits of the largest finite kappa
+    unsigned bits[2];      // max |du|, max |u| of a check inside a pass or in the tile kernel, as floats' bits
+    int tile_err;          // a wait between the tile kernel's CTAs gave up
+    int pad;
+};
+
 struct lbm_grid {
     lbm_params p;
     double nu = 0, S = 1;
@@ -120,27 +129,25 @@ struct lbm_grid {
     int coef_mode = COEF_SCALAR;
     bool has_g = false;
     cudaStream_t stream = nullptr;   // user's stream
-    cudaStream_t cap = nullptr;      // private stream used only for graph capture
+    cudaStream_t cap = nullptr;      // private stream used only for graph capture, made when first needed
     int64_t plane = 0;
     void *buf[2] = {nullptr, nullptr};
     int cur = 0;                     // buf[cur] = post-collision state of the last step
     void *coef = nullptr;
     void *gfield = nullptr;
     double *partials = nullptr;
-    double *result = nullptr;        // device [4]
-    unsigned *flags = nullptr;       // device [2]: error bits, max finite kappa bits
-    double *h_result = nullptr;      // pinned [4]
+    Outcome *outcome = nullptr;      // device
+    Outcome *h_outcome = nullptr;    // pinned, for runs that stop at a tolerance: made when first needed, since it
+                                     // costs 0.28 ms with its release; other calls read once, into the stack
     GridLaunch L{};
     int64_t t = 0;
     int sms = 1;
     bool fused = false;              // several steps per pass (multistep.cu) where a call takes several
     TileGeom tiles{0, 0, 0, 0, 0};   // ntx > 0: a small lattice, stepped in shared memory (tiles.cu)
-    unsigned *check_bits = nullptr;  // a check's maxima inside a pass
-    void *work = nullptr;            // holds partials, result, flags, check_bits, tile_exch and tile_result
+    void *mem = nullptr;             // the one allocation behind every device pointer of the grid
     void *tile_exch = nullptr;       // exchanges between its CTAs
     unsigned tile_base = 0;          // exchanges so far, and more
     unsigned *tile_result = nullptr; // the checks' maxima of one launch, behind the exchanges
-    int *tile_err = nullptr;         // pinned, in h_result: a wait between its CTAs gave up
     struct Graph {
         cudaGraphExec_t exec;
         int kernels;                 // launches it holds
@@ -236,11 +243,11 @@ static cudaError_t enqueue_multi(const lbm_grid *g, int src_idx, int nlev, unsig
 }
 
 // n steps in one launch, the lattice resident in shared memory (tiles.cu), with the checks that fall into them
-// (check_every > 0); *checks: how many. Leaves the newest state in buf[cur]. The last check's maxima come back in
-// h_result as floats' bits.
+// (check_every > 0); *checks: how many. Leaves the newest state in buf[cur], the last check's maxima in the
+// outcome's bits.
 static cudaError_t enqueue_tiles(lbm_grid *g, int n, int check_every, int *checks)
 {
-    TileRun run{n, 0, check_every, g->tile_result, g->tile_exch, g->tile_base, g->tile_err};
+    TileRun run{n, 0, check_every, g->tile_result, g->tile_exch, g->tile_base, &g->outcome->tile_err};
     *checks = 0;
     if (check_every > 0) {
         run.first_check = (int)(check_every - g->t % check_every);
@@ -261,20 +268,30 @@ static cudaError_t enqueue_tiles(lbm_grid *g, int n, int check_every, int *check
         e = launch_tiles(LBM_F32, g->coef_mode, g->has_g, walls, &a, g->tiles, run, g->stream);
     }
     if (e == cudaSuccess && *checks > 0)
-        e = cudaMemcpyAsync(g->h_result + 4, g->tile_result + 2 * (*checks - 1), 2 * sizeof(unsigned),
-                            cudaMemcpyDeviceToHost, g->stream);
+        e = cudaMemcpyAsync(g->outcome->bits, g->tile_result + 2 * (*checks - 1), 2 * sizeof(unsigned),
+                            cudaMemcpyDeviceToDevice, g->stream);
     if (e != cudaSuccess) return e;
     g->tile_base += n / TILE_HALO + 1;
     g->cur = 1 - g->cur;
     return e;
 }
 
-// The residual of a check that left its maxima as floats' bits.
-static double bits_residual(const lbm_grid *g)
+// The outcome of the calls so far, after a synchronisation with the grid's stream.
+static cudaError_t read_outcome(lbm_grid *g, Outcome *o)
+{
+    Outcome *to = g->h_outcome ? g->h_outcome : o;
+    cudaError_t e = cudaMemcpyAsync(to, g->outcome, sizeof *to, cudaMemcpyDeviceToHost, g->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
+    if (e == cudaSuccess && to != o) *o = *to;
+    return e;
+}
+
+// The residual of the last check, which left its maxima in bits or in sums.
+static double residual_of(const Outcome &o, bool as_bits)
 {
     float m[2];
-    std::memcpy(m, g->h_result + 4, sizeof m);
-    const double dmax = m[0], umax = m[1];
+    std::memcpy(m, o.bits, sizeof m);
+    const double dmax = as_bits ? m[0] : o.sums[0], umax = as_bits ? m[1] : o.sums[1];
     return umax > 0.0 ? dmax / umax : dmax;
 }
 
@@ -296,11 +313,12 @@ static lbm_status get_graph(lbm_grid *g, int n, int parity, int check, int pair,
         return LBM_OK;
     }
     cudaGraph_t graph = nullptr;
+    if (!g->cap) LBM_CUDA(cudaStreamCreateWithFlags(&g->cap, cudaStreamNonBlocking));
     LBM_CUDA(cudaStreamBeginCapture(g->cap, cudaStreamCaptureModeThreadLocal));
     cudaError_t err = cudaSuccess;
     int idx = parity, kernels = 0;
     const bool inside = check == CHECK_INSIDE;
-    if (inside) err = cudaMemsetAsync(g->check_bits, 0, 2 * sizeof(unsigned), g->cap);
+    if (inside) err = cudaMemsetAsync(g->outcome->bits, 0, sizeof g->outcome->bits, g->cap);
     for (int left = n; left > 0 && err == cudaSuccess; ++kernels) {
         int take = 1;
         const bool last = inside && left == MULTISTEP_MAX;
@@ -308,17 +326,14 @@ static lbm_status get_graph(lbm_grid *g, int n, int parity, int check, int pair,
             take = inside && !last ? left - MULTISTEP_MAX : left - (pair || check == 1 ? 1 : 0);
             take = take < 1 ? 1 : (take > MULTISTEP_MAX ? MULTISTEP_MAX : take);
         }
-        err = take > 1 ? enqueue_multi(g, idx, take, last ? g->check_bits : nullptr, g->cap) : enqueue_step(g, idx, g->cap);
+        err = take > 1 ? enqueue_multi(g, idx, take, last ? g->outcome->bits : nullptr, g->cap)
+                       : enqueue_step(g, idx, g->cap);
         idx = 1 - idx;
         left -= take;
     }
-    if (inside && err == cudaSuccess)
-        err = cudaMemcpyAsync(g->h_result + 4, g->check_bits, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, g->cap);
     if (check == 1 && err == cudaSuccess) {
         err = enqueue_moments(g, idx, 1 - idx, nullptr, nullptr, nullptr, g->cap);
-        if (err == cudaSuccess) err = launch_reduce_partials(g->partials, g->L.mom_blocks, g->result, g->cap);
-        if (err == cudaSuccess)
-            err = cudaMemcpyAsync(g->h_result, g->result, 4 * sizeof(double), cudaMemcpyDeviceToHost, g->cap);
+        if (err == cudaSuccess) err = launch_reduce_partials(g->partials, g->L.mom_blocks, g->outcome->sums, g->cap);
         kernels += 2;
     }
     cudaError_t e2 = cudaStreamEndCapture(g->cap, &graph);
@@ -447,12 +462,8 @@ static void free_grid(lbm_grid *g)
     if (!g) return;
     for (auto &kv : g->graphs) cudaGraphExecDestroy(kv.second.exec);
     g->graphs.clear();
-    cudaFree(g->buf[0]);
-    cudaFree(g->buf[1]);
-    cudaFree(g->coef);
-    cudaFree(g->gfield);
-    cudaFree(g->work);
-    if (g->h_result) cudaFreeHost(g->h_result);
+    cudaFree(g->mem);
+    if (g->h_outcome) cudaFreeHost(g->h_outcome);
     if (g->cap) cudaStreamDestroy(g->cap);
     cudaGetLastError();
     delete g;
@@ -532,48 +543,46 @@ lbm_status grid_create_impl(const lbm_params *p, const float *kappa_dev, const d
     const int64_t mcap = (int64_t)sms * 2;   // 128 registers: two 256-thread blocks per SM
     g->L.mom_blocks = (int)(mwant < mcap ? (mwant < 1 ? 1 : mwant) : mcap);
 
-    LBM_GRID_CUDA(cudaStreamCreateWithFlags(&g->cap, cudaStreamNonBlocking));
-    LBM_GRID_CUDA(cudaMalloc(&g->buf[0], 9 * g->plane * sb));
-    LBM_GRID_CUDA(cudaMalloc(&g->buf[1], 9 * g->plane * sb));
-    LBM_GRID_CUDA(cudaMalloc(&g->coef, ncoef * g->plane * cb));
-    if (g->has_g) LBM_GRID_CUDA(cudaMalloc(&g->gfield, 2 * g->plane * cb));
-    LBM_GRID_CUDA(cudaMallocHost(&g->h_result, 8 * sizeof(double)));
-    g->tile_err = reinterpret_cast<int *>(g->h_result + 6);
-    *g->tile_err = 0;
     if (g->fused) g->tiles = tile_geometry(p->storage, g->coef_mode, g->has_g, p->nx, p->ny, sms);
-    // one allocation for the reductions' small arrays and the exchanges of the tile kernel; no room for the
-    // latter: stepped in passes over memory
-    const size_t small = 4 * sizeof(double) * (g->L.mom_blocks + 1) + 4 * sizeof(unsigned);     // a multiple of 16
-    const size_t exch = g->tiles.ntx > 0 ? tile_exchange_bytes(n) : 0;
-    if (g->tiles.ntx > 0 &&
-        cudaMalloc(&g->work, small + exch + 2 * sizeof(unsigned) * TILE_CHUNK) != cudaSuccess) {
-        cudaGetLastError();
-        g->work = nullptr;
-        g->tiles.ntx = 0;
+    // One allocation for everything, zeroed in one go: with one each, a memset each, a capture stream and pinned
+    // memory a coarse run of 1250 steps on 256 x 256 took 2.3 ms instead of 1.8. No room for the exchanges of the tile kernel: stepped in passes over memory.
+    auto aligned = [](size_t bytes) { return (bytes + 255) / 256 * 256; };
+    const size_t b_buf = aligned(9 * g->plane * sb), b_coef = aligned(ncoef * g->plane * cb);
+    const size_t b_field = g->has_g ? aligned(2 * g->plane * cb) : 0;
+    const size_t b_small = aligned(4 * sizeof(double) * g->L.mom_blocks + sizeof(Outcome));
+    const size_t base = 2 * b_buf + b_coef + b_field + b_small;
+    size_t exch = 0;
+    if (g->tiles.ntx > 0) {
+        exch = aligned(tile_exchange_bytes(n));
+        if (cudaMalloc(&g->mem, base + exch + 2 * sizeof(unsigned) * TILE_CHUNK) != cudaSuccess) {
+            cudaGetLastError();
+            g->mem = nullptr;
+            g->tiles.ntx = 0;
+            exch = 0;
+        }
     }
-    if (g->tiles.ntx == 0) LBM_GRID_CUDA(cudaMalloc(&g->work, small));
-    g->partials = static_cast<double *>(g->work);
-    g->result = g->partials + 4 * g->L.mom_blocks;
-    g->flags = reinterpret_cast<unsigned *>(g->result + 4);
-    g->check_bits = g->flags + 2;
-    g->tile_exch = reinterpret_cast<char *>(g->work) + small;
-    g->tile_result = reinterpret_cast<unsigned *>(static_cast<char *>(g->tile_exch) + exch);
-    if (g->tiles.ntx > 0) LBM_GRID_CUDA(cudaMemsetAsync(g->tile_exch, 0, exch, g->stream));
+    if (g->tiles.ntx == 0) LBM_GRID_CUDA(cudaMalloc(&g->mem, base));
+    char *m = static_cast<char *>(g->mem);
+    g->buf[0] = m;
+    g->buf[1] = m + b_buf;
+    g->coef = m + 2 * b_buf;
+    if (g->has_g) g->gfield = m + 2 * b_buf + b_coef;
+    g->partials = reinterpret_cast<double *>(m + 2 * b_buf + b_coef + b_field);
+    g->outcome = reinterpret_cast<Outcome *>(g->partials + 4 * g->L.mom_blocks);
+    g->tile_exch = m + base;
+    g->tile_result = reinterpret_cast<unsigned *>(m + base + exch);
 
     cudaStream_t st = g->stream;
     // rest state: deviations are zero in both buffers (state of step -1 and -2)
-    LBM_GRID_CUDA(cudaMemsetAsync(g->buf[0], 0, 9 * g->plane * sb, st));
-    LBM_GRID_CUDA(cudaMemsetAsync(g->buf[1], 0, 9 * g->plane * sb, st));
-    LBM_GRID_CUDA(cudaMemsetAsync(g->coef, 0, ncoef * g->plane * cb, st));
-    LBM_GRID_CUDA(cudaMemsetAsync(g->flags, 0, 2 * sizeof(unsigned), st));
+    LBM_GRID_CUDA(cudaMemsetAsync(m, 0, base + exch, st));
     if (kstar_dev) {
         // The coarse run passes a K* already divided by r^2 when kstar_scale != 1.
         LBM_GRID_CUDA(launch_coef_tensor(p->storage, kstar_dev, g->coef, n, g->plane,
-                                         0.5 * p->eps * g->nu / kstar_scale, g->flags, st));
+                                         0.5 * p->eps * g->nu / kstar_scale, g->outcome->flags, st));
         count_launches(1);
     } else {
-        LBM_GRID_CUDA(launch_coef_scalar(p->storage, kappa_dev, g->coef, n, g->plane, p->eps * g->nu, g->flags,
-                                         g->flags + 1, st));
+        LBM_GRID_CUDA(launch_coef_scalar(p->storage, kappa_dev, g->coef, n, g->plane, p->eps * g->nu, g->outcome->flags,
+                                         g->outcome->flags + 1, st));
         count_launches(1);
     }
     if (g->has_g) {
@@ -581,7 +590,7 @@ lbm_status grid_create_impl(const lbm_params *p, const float *kappa_dev, const d
         count_launches(1);
     }
     unsigned hflags[2] = {0, 0};
-    LBM_GRID_CUDA(cudaMemcpyAsync(hflags, g->flags, sizeof hflags, cudaMemcpyDeviceToHost, st));
+    LBM_GRID_CUDA(cudaMemcpyAsync(hflags, g->outcome->flags, sizeof hflags, cudaMemcpyDeviceToHost, st));
     LBM_GRID_CUDA(cudaStreamSynchronize(st));
     if (hflags[0] & 1u) return bail(fail(LBM_EINVAL, kstar_dev ? "K* has non-finite entries"
                                                                  : "kappa has negative or NaN entries"));
@@ -652,10 +661,13 @@ lbm_status lbm_step(lbm_grid *g, int64_t max_steps, double tol_rel, int32_t chec
     if (!std::isfinite(tol_rel)) return fail(LBM_EINVAL, "tol_rel must be finite");
     if (tol_rel > 0.0 && check_every == 0) return fail(LBM_EINVAL, "tol_rel > 0 needs check_every > 0");
     DeviceGuard dg(g->dev);
+    if (tol_rel > 0.0 && !g->h_outcome) LBM_CUDA(cudaMallocHost(&g->h_outcome, sizeof *g->h_outcome));
     const int CHUNK = 1024;
     int64_t left = max_steps, done = 0;
     double resid = -1.0;
     bool converged = false, checked = false, as_bits = false;       // as_bits: how the last check left its result
+    bool tiled = false;
+    Outcome o{};
     while (left > 0) {
         // one launch of the tile kernel runs up to the next value the host needs
         int64_t m = left < TILE_CHUNK ? left : TILE_CHUNK;
@@ -670,15 +682,16 @@ lbm_status lbm_step(lbm_grid *g, int64_t max_steps, double tol_rel, int32_t chec
             }
             LBM_CUDA(e);
             count_launches(1);
+            tiled = true;
             g->t += m;
             done += m;
             left -= m;
             if (checks == 0) continue;
             checked = as_bits = true;
             if (tol_rel > 0.0) {
-                LBM_CUDA(cudaStreamSynchronize(g->stream));
-                resid = bits_residual(g);
-                if (resid <= tol_rel) {
+                LBM_CUDA(read_outcome(g, &o));
+                resid = residual_of(o, true);
+                if (o.tile_err || resid <= tol_rel) {
                     converged = true;
                     break;
                 }
@@ -710,9 +723,8 @@ lbm_status lbm_step(lbm_grid *g, int64_t max_steps, double tol_rel, int32_t chec
             checked = true;
             as_bits = check == CHECK_INSIDE;
             if (tol_rel > 0.0) {      // the stop test needs the value now; otherwise read it at the end
-                LBM_CUDA(cudaStreamSynchronize(g->stream));
-                const double dmax = g->h_result[0], umax = g->h_result[1];
-                resid = umax > 0.0 ? dmax / umax : dmax;
+                LBM_CUDA(read_outcome(g, &o));
+                resid = residual_of(o, false);
                 if (resid <= tol_rel) {
                     converged = true;
                     break;
@@ -720,17 +732,16 @@ lbm_status lbm_step(lbm_grid *g, int64_t max_steps, double tol_rel, int32_t chec
             }
         }
     }
-    LBM_CUDA(cudaStreamSynchronize(g->stream));
-    if (*(volatile int *)g->tile_err) {                      // the state is not valid any more
-        *g->tile_err = 0;
+    if (tiled || (checked && tol_rel <= 0.0)) {
+        LBM_CUDA(read_outcome(g, &o));
+    } else {
+        LBM_CUDA(cudaStreamSynchronize(g->stream));
+    }
+    if (o.tile_err) {                                        // the state is not valid any more
+        cudaMemsetAsync(&g->outcome->tile_err, 0, sizeof(int), g->stream);
         return fail(LBM_ECUDA, "a wait between the tiles of the lattice gave up");
     }
-    if (checked && tol_rel <= 0.0 && as_bits) {
-        resid = bits_residual(g);
-    } else if (checked && tol_rel <= 0.0) {
-        const double dmax = g->h_result[0], umax = g->h_result[1];
-        resid = umax > 0.0 ? dmax / umax : dmax;
-    }
+    if (checked && tol_rel <= 0.0) resid = residual_of(o, as_bits);
     if (steps_done) *steps_done = done;
     if (residual) *residual = resid;
     if (tol_rel > 0.0 && !converged)
@@ -756,13 +767,13 @@ lbm_status lbm_mean_velocity(lbm_grid *g, double out_mean_uv[2])
     if (!g || !out_mean_uv) return fail(LBM_EINVAL, "grid or output is NULL");
     DeviceGuard dg(g->dev);
     LBM_CUDA(enqueue_moments(g, g->cur, -1, nullptr, nullptr, nullptr, g->stream));
-    LBM_CUDA(launch_reduce_partials(g->partials, g->L.mom_blocks, g->result, g->stream));
+    LBM_CUDA(launch_reduce_partials(g->partials, g->L.mom_blocks, g->outcome->sums, g->stream));
     count_launches(2);
-    LBM_CUDA(cudaMemcpyAsync(g->h_result, g->result, 4 * sizeof(double), cudaMemcpyDeviceToHost, g->stream));
-    LBM_CUDA(cudaStreamSynchronize(g->stream));
+    Outcome o;
+    LBM_CUDA(read_outcome(g, &o));
     const double n = (double)g->p.nx * g->p.ny;
-    out_mean_uv[0] = g->h_result[2] / n;
-    out_mean_uv[1] = g->h_result[3] / n;
+    out_mean_uv[0] = o.sums[2] / n;
+    out_mean_uv[1] = o.sums[3] / n;
     return LBM_OK;
 }
 

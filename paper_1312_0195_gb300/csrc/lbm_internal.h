@@ -91,10 +91,10 @@ struct TileGeom {
     int ctas;         // CTAs, two tiles each
 };
 TileGeom tile_geometry(int storage, int coef_mode, bool gfield, int nx, int ny, int sms);
-// Steps of a launch at least (more than TILE_HALO: an exchange has to take place). Filling shared memory and writing
-// it back costs 15 to 20 us: a call of 8 steps took 23 us at 128 x 64 and 39 us at 500 x 500, in passes of four 25 and
-// 32 us; one of 12 steps 27 and 48 us against 33 and 43 us, one of 24 steps 38 and 73 us against 48 and 75 us.
-constexpr int TILES_FROM = 12;
+// Steps of a launch at least (more than TILE_HALO: an exchange has to take place). Filling shared memory, writing it
+// back and reading the outcome cost about 20 us. Microseconds of a call here / in passes of four: 12 steps 31 / 33 at
+// 128 x 64, 46 / 47 at 517 x 389, 52 / 44 at 500 x 500, the largest; 16 steps 60 / 55 and 24 steps 77 / 76 there.
+constexpr int TILES_FROM = 16;
 constexpr size_t tile_exchange_bytes(int64_t cells) { return (size_t)cells * 2 * 3 * 16; }
 // One launch: `steps` steps from the state in src, with the residual's maxima (bits of max |du| and max |u|) after
 // step first_check and every check_every-th step on (check_every = 0: none) raised in result[2 c], result[2 c + 1] for
