@@ -545,7 +545,8 @@ lbm_status grid_create_impl(const lbm_params *p, const float *kappa_dev, const d
 
     if (g->fused) g->tiles = tile_geometry(p->storage, g->coef_mode, g->has_g, p->nx, p->ny, sms);
     // One allocation for everything, zeroed in one go: with one each, a memset each, a capture stream and pinned
-    // memory a coarse run of 1250 steps on 256 x 256 took 2.3 ms instead of 1.8. No room for the exchanges of the tile kernel: stepped in passes over memory.
+    // memory a coarse run of 1250 steps on 256 x 256 took 2.3 ms instead of 1.8. No room for the exchanges of the
+    // tile kernel: stepped in passes over memory.
     auto aligned = [](size_t bytes) { return (bytes + 255) / 256 * 256; };
     const size_t b_buf = aligned(9 * g->plane * sb), b_coef = aligned(ncoef * g->plane * cb);
     const size_t b_field = g->has_g ? aligned(2 * g->plane * cb) : 0;
