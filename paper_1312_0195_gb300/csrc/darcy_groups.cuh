@@ -249,6 +249,9 @@ __global__ void __launch_bounds__(RG_THREADS, 1) darcy_group_kernel(const float 
             if (mine && warp == q.w0 && q.row == 0 && q.col == 0)
                 cw[leaf] = make_float4((float)log(qx / (s * s)), 1.0f, (float)log(qy / (s * s)), 1.0f);
         }
+        // every warp of the group has read that the list is empty before a smaller group of the next class, which
+        // some of them may already belong to, puts its leaves into the same words
+        group_sync(q.group, q.w0);
     }
 }
 

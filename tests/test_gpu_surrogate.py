@@ -406,3 +406,22 @@ def test_darcy_base_of_every_side_matches_oracle(counts):
         c, _ = _base_from_predict(sur, x, 3)
     ref = np.array([S.target_base(lk.astype(np.float32).astype(np.float64), 3) for lk in leaves])
     np.testing.assert_allclose(c, ref[:, [0, 2]], rtol=0, atol=3e-5)
+
+
+@pytest.mark.parametrize("counts", [{64: 1, 4: 200}, {64: 153, 32: 9, 16: 5, 8: 3, 4: 1}, {32: 1, 16: 700, 8: 1}])
+def test_darcy_base_does_not_depend_on_the_other_sides_of_the_batch(counts):
+    """Groups of warps split when a side's list is empty, and go on to the next side one by one. A leaf's base is the
+    same bits whatever else is in the batch, over and over: alone with its own side, and mixed with the others."""
+    lbm = _lbm()
+    rng = np.random.default_rng(23)
+    leaves = [rng.normal(-4.0, 1.0) + synth.gaussian_random_field(s, s, 2.0, seed=100 * s + i % 7)
+              for s, n in counts.items() for i in range(n)]
+    leaves = [leaves[i] for i in rng.permutation(len(leaves))]
+    x = _inputs(len(leaves), 0, leaves)
+    side = np.array([lk.shape[0] for lk in leaves])
+    ref = np.zeros((len(leaves), 2))
+    with lbm.Surrogate(1, 0) as sur:
+        for s in counts:
+            ref[side == s] = _base_from_predict(sur, x[side == s], 3)[0]
+        for _ in range(20):
+            np.testing.assert_array_equal(_base_from_predict(sur, x, 3)[0], ref)
