@@ -87,6 +87,16 @@ struct Pair3Shared {
 };
 inline size_t pair3_smem_bytes(int ps) { return sizeof(Pair3Shared) + (size_t)ps * Q19 * sizeof(float2); }
 
+// Past the wall-clock limit: the jobs nobody has taken are abandoned too (LBM_ETIMEOUT, no K*, 0 steps).
+__device__ __noinline__ void abandon_queue(const Clu3Args<float> &a, int *head)
+{
+    for (int j; (j = atomicAdd(head, 1)) < a.njobs;) {
+        const int leaf = a.ids[j / 3];
+        for (int i = 0; i < 3; ++i) a.keff[9 * (int64_t)leaf + 3 * i + j % 3] = __longlong_as_double(0x7ff8000000000000LL);
+        atomicMax(&a.status[leaf], (int)LBM_ETIMEOUT);
+    }
+}
+
 // a.njobs jobs from the queue *head (zeroed), a.s^3 cells each, over as many clusters as are resident.
 template <int PS>
 __global__ void __launch_bounds__(CP3_THREADS, 1) local3d_pair_kernel(Clu3Args<float> a, int *head)
@@ -270,6 +280,7 @@ __global__ void __launch_bounds__(CP3_THREADS, 1) local3d_pair_kernel(Clu3Args<f
                 for (int i = 0; i < 3; ++i) a.keff[9 * (int64_t)leaf[k] + 3 * i + drive[k]] = a.nu_over_g * u[i];   // Eq. 17
                 if (a.steps) a.steps[3 * (int64_t)leaf[k] + drive[k]] = (int)t;
                 if (st != LBM_OK) atomicMax(&a.status[leaf[k]], st);
+                if (abort_now) abandon_queue(a, head);
                 sh.job[k] = abort_now ? INT_MAX : atomicAdd(head, 1);
             }
             refill[k] = true;

@@ -344,3 +344,24 @@ def test_local_keff3_two_jobs_a_cluster_match_oracle(sides, tau, steps, k):
         cube = kap[z0:z0 + s, y0:y0 + s, x0:x0 + s].astype(np.float64)
         ref = oracle.local_keff3(cube, tau, 0.1, 0.9, 1e-6, tol=0.0, max_steps=steps, check_every=k)["keff"]
         np.testing.assert_allclose(ke[i], ref, rtol=0, atol=1e-5 * np.abs(np.diag(ref)).max())
+
+
+def test_local_keff3_time_limit_reaches_jobs_still_in_the_queue():
+    """Past the wall-clock limit no leaf is reported as solved: neither the jobs that run nor those that wait in
+    either size's queue (512 cubes of 8 and 125 of 12 cells, several times what the chip holds at once)."""
+    import torch
+    lbm = _lbm()
+    kap = _field(64, 64, 64, seed=80)
+    leaves = [(x, y, z, s) for s in (8, 12) for z in range(0, 65 - s, s) for y in range(0, 65 - s, s)
+              for x in range(0, 65 - s, s)]
+    try:
+        lbm.lbm_set_time_limit(2e-4)
+        ke, st, steps, worst = gpu_keff3(kap, leaves, 1.0, 1.0 / 6.0, 1.0, 1e-6, 1e-14, 10_000_000)
+        assert worst == lbm.LBM_ETIMEOUT
+        assert (st == lbm.LBM_ETIMEOUT).all()
+        assert (np.isnan(ke).all(axis=1) == (steps == 0)).all()
+        _, n_notconv, worst = lbm.lbm3d_upscale(lbm.Params3D(nx=64, ny=64, nz=64, tau=1.0), torch.from_numpy(kap).cuda(), 8,
+                                                1e-6, 1e-14, 10_000_000)
+        assert worst == lbm.LBM_ETIMEOUT and n_notconv == 512
+    finally:
+        lbm.lbm_set_time_limit(600.0)
