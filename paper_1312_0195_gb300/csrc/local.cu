@@ -1060,6 +1060,38 @@ __global__ void lg_finish_kernel(int64_t n, const int *pos, const float *kuni, c
     for (int q = 0; q < 4; ++q) keff[4 * i + q] = k[q];
 }
 
+// Past the wall-clock limit: the jobs that no CTA has taken are abandoned too (LBM_ETIMEOUT, NaN, 0 steps). After the
+// solvers, whose loops have no registers to spare for it. reg_blocks: CTAs of the register solver, 0 if it did not
+// run; it deals the first jobs of its first class out without the queue.
+__global__ void __launch_bounds__(256) abandon_kernel(LocalArgs a, int reg_blocks)
+{
+    if (!*a.abort_flag) return;
+    const double nan = __longlong_as_double(0x7ff8000000000000LL);
+    const int nclass = a.table ? (a.table[DT_BAD] ? 0 : a.table[DT_NCLASS]) : a.nclass;
+    for (int cls = 0; cls < nclass; ++cls) {
+        const int s = a.table ? a.table[DT_SIZE + cls] : a.class_size[cls];
+        const int qbeg = a.table ? a.table[DT_OFF + cls] : a.class_off[cls];
+        const int qend = a.table ? a.table[DT_OFF + cls + 1] : a.class_off[cls + 1];
+        int taken = a.heads[cls];
+        if (reg_blocks > 0 && reg_side(s)) {
+            const RegGeo q = reg_geometry(s, 0, 0);
+            taken += reg_blocks * (RG_WARPS / q.group) * q.jobs;
+            reg_blocks = 0;
+        }
+        for (int i = qbeg + taken + threadIdx.x; i < qend; i += blockDim.x) {
+            const int leaf = a.jobs[i] >> 1, drive = a.jobs[i] & 1;
+            if (a.lg_win) {
+                for (int k = 0; k < 4; ++k) a.lg_win[4 * (2 * (int64_t)leaf + drive) + k] = nan;
+            } else {
+                a.keff[4 * (int64_t)leaf + drive] = nan;
+                a.keff[4 * (int64_t)leaf + 2 + drive] = nan;
+            }
+            atomicMax(&a.status[leaf], (int)LBM_ETIMEOUT);
+            atomicMax(a.worst, (int)LBM_ETIMEOUT);
+        }
+    }
+}
+
 // Launches the solvers of a batch on `blocks` CTAs: from rest in FP32, sides that are multiples of 4
 // go to the register solver (1.2 to 2.3 times the rate of the shared-memory one at every such side, see
 // local_reg.cuh) and the rest to the shared-memory one; everything else to the latter.
@@ -1086,6 +1118,8 @@ cudaError_t launch_solvers(LocalArgs &a, bool f64, double tau, bool lg, int bloc
         kern<<<blocks, LOCAL_THREADS, smem, st>>>(a);
         count_launches(1);
     }
+    abandon_kernel<<<1, 256, 0, st>>>(a, use_reg && reg ? blocks : 0);
+    count_launches(1);
     return cudaGetLastError();
 }
 

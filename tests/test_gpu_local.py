@@ -350,3 +350,24 @@ def test_every_side_of_the_register_solver_matches_oracle(tau, steps, k):
     for i in range(len(leaves)):
         ref = oracle_keff(kap, leaves[i], tau, 0.1, 0.9, 1e-6, 0.0, steps, k=k)
         assert_keff_close(ke[i], ref["keff"], 1e-4)
+
+
+@pytest.mark.parametrize("storage,warm", [(0, 0), (2, 0), (0, 1)])
+def test_time_limit_reaches_jobs_still_in_the_queue(storage, warm):
+    """Past the wall-clock limit no leaf is reported as solved: neither the jobs that run nor those that wait in a
+    size's queue. Sides of the register solver (32, 8) and of the shared-memory one (30, 7), from rest and from the
+    Darcy state, several times what the chip holds at once."""
+    import torch
+    lbm = _lbm()
+    kap = torch.from_numpy(synth.lognormal_kappa(512, 512, 8.0, 1.0, seed=24).astype(np.float32)).cuda()
+    leaves = np.concatenate([synth.uniform_leaves(512 // s * s, 512 // s * s, s) for s in (32, 30, 8, 7)] * 4)
+    p = lbm.Params(nx=512, ny=512, tau=1.0, storage=storage, warm_start=warm)
+    try:
+        lbm.lbm_set_time_limit(2e-4)
+        ke, st, steps, worst = lbm.local_keff(p, kap, torch.from_numpy(leaves.astype(np.int32)).cuda(), 1e-6, 1e-14,
+                                              10_000_000, 64)
+        assert worst == lbm.LBM_ETIMEOUT
+        assert (st == lbm.LBM_ETIMEOUT).all()
+        assert torch.isnan(ke.reshape(-1, 2, 2)[:, 0, :][steps == 0]).all()
+    finally:
+        lbm.lbm_set_time_limit(600.0)
