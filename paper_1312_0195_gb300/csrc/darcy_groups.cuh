@@ -5,15 +5,17 @@
 // solved at once: they share the matrix, and the two right-hand sides are the lanes of packed f32x2 operands.
 // A thread holds a block of 4 rows x 2 columns (leaf_groups.cuh): pressure, residual, direction (48
 // registers), faces and 1 / diagonal (24). An iteration needs the direction's neighbours along x from the
-// neighbouring lanes, along y from shared memory at the block's edges only, and three sums over the leaf's
-// group of warps: the eight terms of a thread as two chains of four, the threads of a warp and the warps by
-// butterflies, all in FP32 (13 roundings at most on the way of a term; the one-CTA-per-leaf solver this
-// replaces rounded 16 times in FP32 before its FP64 sums, and its FP64 butterflies and per-cell index
-// divisions bounded it).
+// neighbouring lanes, along y from shared memory at the block's edges only, and sums over the leaf's group of
+// warps: the eight terms of a thread as two chains of four in FP32, everything across threads in pairs of floats (a
+// rounded sum and its error, about 46 bits), alpha and beta from those pairs. FP64 sums would keep the pipe's two lanes
+// busy for 1500 clocks an iteration of a 64-cell leaf. Pairs cost 5 % over plain FP32 sums, because a lane that takes
+// half of its partner's values gives away the other half of its own: four sums over a warp take 6 additions, not 20.
+// The faces are scaled by a power of two, so that squares of residuals stay inside FP32's range at any unit of K: with
+// unscaled faces and FP32 sums log K* was 2e-4 off at K around 1e-20 and wrong in the first digit at 6e17.
 //
-// Measured: a 512 x 512 quadtree's leaves (sigma 1) 13.2 -> 1.4 ms; surrogate inference on a 1024 x 1024
-// quadtree 31.2 -> 9.5 ms, the solves in it 22.4 -> 0.6. The largest leaf's iterations, a chain of three
-// barriers and two reductions each, are what remains.
+// Measured: the leaves of a 512 x 512 quadtree (sigma 1) 12.2 ms with a warp or a CTA per leaf and FP64 sums, 0.625 ms
+// here (0.594 with FP32 sums); surrogate inference on a 1024 x 1024 quadtree 29.0 -> 7.5 ms. The largest leaf's
+// iterations, a chain of three barriers and two reductions each, are what remains.
 #pragma once
 
 #include "leaf_groups.cuh"
@@ -22,9 +24,10 @@
 namespace lbm {
 namespace sur {
 
-// Square of the relative residual, 5e-6: half of what the FP64-summed solver stopped at, which makes up for the
-// FP32 sums. Against 64-bit solves the mean error of log K* is what it was (1e-7 to 5e-7 at sigma <= 2, any
-// scale of K) and on 64-cell leaves at sigma 3 half of it (3.0e-5 against 6.5e-5).
+// Square of the relative residual, 5e-6: half of what the solver with FP64 sums (darcy_leaf) stops at, since a thread's
+// eight terms are a longer chain in FP32 than there on small leaves. Mean error of log K* against 64-bit solves, there /
+// here: 9e-8 both at sigma <= 1 (the result's own rounding); at sigma 3 1.4e-6 / 1.3e-6 at side 8, 2.5e-6 / 2.4e-6 at 16,
+// 5.2e-6 / 3.1e-6 at 32, 3.0e-6 / 2.8e-6 at 64, and 5.1e-7 / 5.4e-7 at side 4.
 constexpr float DG_STOP = 2.5e-11f;
 constexpr int DG_CLASSES = 5;                // sides 64, 32, 16, 8, 4
 __host__ __device__ constexpr int dg_side(int c) { return 64 >> c; }
@@ -38,7 +41,8 @@ inline size_t darcy_scratch_ints(int n) { return DG_HEADER + (size_t)DG_LISTS * 
 struct DarcyShared {
     double k[RG_WARPS * RG_WCELLS];          // permeability while a leaf is set up
     float4 edge[RG_WARPS][2][32];            // a block's bottom and top row: (column, column + 1) x (drive x, drive y)
-    float2 sum[3][RG_WARPS];                 // a warp's part of a sum over its group
+    float2 sum4[4][RG_WARPS], sum2[2][RG_WARPS];   // a warp's part of sums over its group
+    float kmax[RG_WARPS];
     double flux[2][RG_WARPS];
     int leaf[RG_WARPS][RG_JOBS];
 };
@@ -53,6 +57,43 @@ __global__ void __launch_bounds__(256) darcy_classify_kernel(const float *x, int
             if (s == dg_side(k)) c = k;
         scratch[DG_HEADER + (int64_t)c * n + atomicAdd(&scratch[c], 1)] = i;
     }
+}
+
+// A sum carried to twice FP32's precision: hi + lo.
+struct Two {
+    float hi, lo;
+};
+// a + b without error (Knuth's two-sum); the same bits whichever comes first
+__device__ __forceinline__ Two two_sum(float a, float b)
+{
+    const float s = a + b, t = s - a;
+    return Two{s, (a - (s - t)) + (b - t)};
+}
+// the low parts are not carried over into the high one: their sum's rounding is 2^-24 of 2^-24
+__device__ __forceinline__ Two two_add(Two a, Two b)
+{
+    const Two s = two_sum(a.hi, b.hi);
+    return Two{s.hi, s.lo + (a.lo + b.lo)};
+}
+__device__ __forceinline__ Two two_norm(Two a)
+{
+    const float s = a.hi + a.lo;
+    return Two{s, a.lo - (s - a.hi)};
+}
+__device__ __forceinline__ Two two_shfl_xor(Two a, int off)
+{
+    return Two{__shfl_xor_sync(0xffffffffu, a.hi, off), __shfl_xor_sync(0xffffffffu, a.lo, off)};
+}
+__device__ __forceinline__ Two two_shfl(Two a, int from)
+{
+    return Two{__shfl_sync(0xffffffffu, a.hi, from), __shfl_sync(0xffffffffu, a.lo, from)};
+}
+// a / b, rounded to FP32 once (up to about 2^-40)
+__device__ __forceinline__ float two_div(Two a, Two b)
+{
+    const float q = a.hi / b.hi;
+    const float r = fmaf(-q, b.hi, a.hi) + fmaf(-q, b.lo, a.lo);
+    return q + __fdividef(r, b.hi);
 }
 
 __global__ void __launch_bounds__(RG_THREADS, 1) darcy_group_kernel(const float *x, int n, int *scratch, float4 *cw)
@@ -74,18 +115,47 @@ __global__ void __launch_bounds__(RG_THREADS, 1) darcy_group_kernel(const float 
         auto from_left = [&](float2 v) {
             return make_float2(__shfl_sync(0xffffffffu, v.x, q.left), __shfl_sync(0xffffffffu, v.y, q.left));
         };
-        // a sum over the leaf, the same bits in each of its threads
-        auto total = [&](float2 v, int slot) {
-            for (int off = span / 2; off > 0; off >>= 1)
-                v = add2(v, make_float2(__shfl_xor_sync(0xffffffffu, v.x, off), __shfl_xor_sync(0xffffffffu, v.y, off)));
-            if (q.group > 1) {
-                if (lane == 0) sh.sum[slot][warp] = v;
-                group_sync(q.group, q.w0);
-                v = sh.sum[slot][q.w0 + (lane & (q.group - 1))];
-                for (int off = q.group / 2; off > 0; off >>= 1)
-                    v = add2(v, make_float2(__shfl_xor_sync(0xffffffffu, v.x, off), __shfl_xor_sync(0xffffffffu, v.y, off)));
+        // The sums over the leaf of (a.x, a.y, b.x, b.y), a and b each as two addends, and of c, the same bits in each
+        // of its threads. A lane keeps half of what it holds and gives the other half to its partner, until it
+        // holds one sum's part (offsets span / 2 and span / 4; a span of 2 lanes stops at two sums each).
+        auto totals4 = [&](float2 a0, float2 a1, float2 b0, float2 b1, Two (&t)[4]) {
+            Two v[4] = {two_sum(a0.x, a1.x), two_sum(a0.y, a1.y), two_sum(b0.x, b1.x), two_sum(b0.y, b1.y)};
+            const int o1 = span / 2, o2 = span / 4;
+            const bool up1 = lane & o1, up2 = lane & o2;
+            for (int i = 0; i < 2; ++i) v[i] = two_add(up1 ? v[i + 2] : v[i], two_shfl_xor(up1 ? v[i] : v[i + 2], o1));
+            if (span > 2) {
+                v[0] = two_add(up2 ? v[1] : v[0], two_shfl_xor(up2 ? v[0] : v[1], o2));
+                for (int off = span / 8; off > 0; off >>= 1) v[0] = two_add(v[0], two_shfl_xor(v[0], off));
             }
-            return v;
+            if (q.group > 1) {                                   // span = 32: lanes 8 k .. 8 k + 7 hold sum k
+                if ((lane & 7) == 0) sh.sum4[lane >> 3][warp] = make_float2(v[0].hi, v[0].lo);
+                group_sync(q.group, q.w0);
+                const int w = lane & 7;
+                const float2 *part = sh.sum4[lane >> 3] + q.w0;
+                const float2 p0 = w < q.group ? part[w] : dup2(0.0f), p1 = w + 8 < q.group ? part[w + 8] : dup2(0.0f);
+                v[0] = two_add(Two{p0.x, p0.y}, Two{p1.x, p1.y});
+                for (int off = 4; off > 0; off >>= 1) v[0] = two_add(v[0], two_shfl_xor(v[0], off));
+            }
+            const int base = lane & ~(span - 1);
+            for (int k = 0; k < 4; ++k)
+                t[k] = two_norm(two_shfl(span > 2 || !(k & 1) ? v[0] : v[1], base + (k >> 1) * o1 + (k & 1) * o2));
+        };
+        auto totals2 = [&](float2 c0, float2 c1, Two (&t)[2]) {
+            Two v[2] = {two_sum(c0.x, c1.x), two_sum(c0.y, c1.y)};
+            const int o1 = span / 2;
+            const bool up = lane & o1;
+            v[0] = two_add(up ? v[1] : v[0], two_shfl_xor(up ? v[0] : v[1], o1));
+            for (int off = span / 4; off > 0; off >>= 1) v[0] = two_add(v[0], two_shfl_xor(v[0], off));
+            if (q.group > 1) {
+                if ((lane & 15) == 0) sh.sum2[lane >> 4][warp] = make_float2(v[0].hi, v[0].lo);
+                group_sync(q.group, q.w0);
+                const int w = lane & 15;
+                const float2 p = w < q.group ? sh.sum2[lane >> 4][q.w0 + w] : dup2(0.0f);
+                v[0] = Two{p.x, p.y};
+                for (int off = 8; off > 0; off >>= 1) v[0] = two_add(v[0], two_shfl_xor(v[0], off));
+            }
+            const int base = lane & ~(span - 1);
+            for (int k = 0; k < 2; ++k) t[k] = two_norm(two_shfl(v[0], base + k * o1));
         };
         for (;;) {
             group_sync(q.group, q.w0);                           // the previous leaf's reads are done
@@ -112,7 +182,7 @@ __global__ void __launch_bounds__(RG_THREADS, 1) darcy_group_kernel(const float 
             group_sync(q.group, q.w0);
             float kx[RG_ROWS][2], ky[RG_ROWS][2], kb[2], idg[RG_ROWS][2];    // kb: the faces below the block
             float2 p[RG_ROWS][2], res[RG_ROWS][2], d[RG_ROWS][2], ad[RG_ROWS][2];
-            float2 rr = dup2(0.0f), rz = dup2(0.0f);
+            Two rz[2];
 #pragma unroll
             for (int r = 0; r < RG_ROWS; ++r)
 #pragma unroll
@@ -133,7 +203,31 @@ __global__ void __launch_bounds__(RG_THREADS, 1) darcy_group_kernel(const float 
                     }
                 for (int c = 0; c < 2; ++c) kb[c] = harmonic2f(at(q.row - 1, q.col + c), at(q.row, q.col + c));
             }
+            // the faces over the power of two at the leaf's largest one, so that squares of residuals keep clear of
+            // FP32's ends whatever the unit of K (exact, and pressures do not depend on it); K* takes it back
+            float top = 0.0f;
+#pragma unroll
+            for (int r = 0; r < RG_ROWS; ++r) top = fmaxf(top, fmaxf(fmaxf(kx[r][0], kx[r][1]), fmaxf(ky[r][0], ky[r][1])));
+            for (int off = span / 2; off > 0; off >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, off));
+            if (q.group > 1) {
+                if (lane == 0) sh.kmax[warp] = top;
+                group_sync(q.group, q.w0);
+                for (int w = 0; w < q.group; ++w) top = fmaxf(top, sh.kmax[q.w0 + w]);
+            }
+            int unit = (__float_as_int(top) >> 23) - 127;
+            unit = unit > 127 ? 0 : min(max(unit, -126), 126);       // an infinite face: as it is
+            const float scale = __int_as_float((127 - unit) << 23);
+#pragma unroll
+            for (int r = 0; r < RG_ROWS; ++r)
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    kx[r][c] *= scale;
+                    ky[r][c] *= scale;
+                }
+            kb[0] *= scale;
+            kb[1] *= scale;
             // start: p = 0, r = b (face behind minus face ahead along the drive), d = r / diagonal
+            float2 r0 = dup2(0.0f), r1 = dup2(0.0f), g0 = dup2(0.0f), g1 = dup2(0.0f);
 #pragma unroll
             for (int r = 0; r < RG_ROWS; ++r) {
                 const float kl = __shfl_sync(0xffffffffu, kx[r][1], q.left);
@@ -144,14 +238,16 @@ __global__ void __launch_bounds__(RG_THREADS, 1) darcy_group_kernel(const float 
                     idg[r][c] = dg > 0.0f ? 1.0f / dg : 0.0f;
                     res[r][c] = mine ? make_float2(xl - kx[r][c], yb - ky[r][c]) : dup2(0.0f);
                     d[r][c] = mul2(res[r][c], dup2(idg[r][c]));
-                    rr = fma2(res[r][c], res[r][c], rr);
-                    rz = fma2(res[r][c], d[r][c], rz);
+                    (c == 0 ? r0 : r1) = fma2(res[r][c], res[r][c], c == 0 ? r0 : r1);
+                    (c == 0 ? g0 : g1) = fma2(res[r][c], d[r][c], c == 0 ? g0 : g1);
                 }
             }
-            rr = total(rr, 0);
-            rz = total(rz, 1);
-            const float2 stop = mul2(dup2(DG_STOP), rr);
-            bool on0 = mine && rr.x > stop.x, on1 = mine && rr.y > stop.y;
+            Two t[4];                                            // r . r of both drives, r . z of both drives
+            totals4(r0, r1, g0, g1, t);
+            rz[0] = t[2];
+            rz[1] = t[3];
+            const float2 stop = mul2(dup2(DG_STOP), make_float2(t[0].hi, t[1].hi));
+            bool on0 = mine && t[0].hi > stop.x, on1 = mine && t[1].hi > stop.y;
             auto publish = [&](const float2 (&v)[RG_ROWS][2]) {
                 sh.edge[warp][0][lane] = make_float4(v[0][0].x, v[0][0].y, v[0][1].x, v[0][1].y);
                 sh.edge[warp][1][lane] = make_float4(v[RG_ROWS - 1][0].x, v[RG_ROWS - 1][0].y, v[RG_ROWS - 1][1].x,
@@ -183,10 +279,11 @@ __global__ void __launch_bounds__(RG_THREADS, 1) darcy_group_kernel(const float 
                     t0 = fma2(d[r][0], ad[r][0], t0);
                     t1 = fma2(d[r][1], ad[r][1], t1);
                 }
-                const float2 dad = total(add2(t0, t1), 2);
-                on0 = on0 && dad.x > 0.0f;                       // else a direction in the null space
-                on1 = on1 && dad.y > 0.0f;
-                const float2 al = make_float2(on0 ? rz.x / dad.x : 0.0f, on1 ? rz.y / dad.y : 0.0f);
+                Two dad[2];
+                totals2(t0, t1, dad);
+                on0 = on0 && dad[0].hi > 0.0f;                   // else a direction in the null space
+                on1 = on1 && dad[1].hi > 0.0f;
+                const float2 al = make_float2(on0 ? two_div(rz[0], dad[0]) : 0.0f, on1 ? two_div(rz[1], dad[1]) : 0.0f);
                 const float2 nal = make_float2(-al.x, -al.y);
                 float2 a0 = dup2(0.0f), a1 = dup2(0.0f), z0 = dup2(0.0f), z1 = dup2(0.0f);
 #pragma unroll
@@ -202,12 +299,12 @@ __global__ void __launch_bounds__(RG_THREADS, 1) darcy_group_kernel(const float 
                     z0 = fma2(s0, dup2(idg[r][0]), z0);
                     z1 = fma2(s1, dup2(idg[r][1]), z1);
                 }
-                rr = total(add2(a0, a1), 0);
-                const float2 rz2 = total(add2(z0, z1), 1);
-                const float2 be = make_float2(on0 ? rz2.x / rz.x : 0.0f, on1 ? rz2.y / rz.y : 0.0f);
-                rz = rz2;
-                on0 = on0 && rr.x > stop.x;
-                on1 = on1 && rr.y > stop.y;
+                totals4(a0, a1, z0, z1, t);
+                const float2 be = make_float2(on0 ? two_div(t[2], rz[0]) : 0.0f, on1 ? two_div(t[3], rz[1]) : 0.0f);
+                rz[0] = t[2];
+                rz[1] = t[3];
+                on0 = on0 && t[0].hi > stop.x;
+                on1 = on1 && t[1].hi > stop.y;
 #pragma unroll
                 for (int r = 0; r < RG_ROWS; ++r)
 #pragma unroll
@@ -218,16 +315,15 @@ __global__ void __launch_bounds__(RG_THREADS, 1) darcy_group_kernel(const float 
             publish(p);
             group_sync(q.group, q.w0);
             const float4 above = sh.edge[ta >> 5][0][ta & 31];
-            float fx = 0.0f, fy = 0.0f;
+            double qx = 0.0, qy = 0.0;
 #pragma unroll
             for (int r = 0; r < RG_ROWS; ++r) {
                 const float pr = __shfl_sync(0xffffffffu, p[r][0].x, q.right);
-                fx += kx[r][0] * (p[r][0].x - p[r][1].x + 1.0f);
-                fx += kx[r][1] * (p[r][1].x - pr + 1.0f);
-                fy += ky[r][0] * (p[r][0].y - (r < RG_ROWS - 1 ? p[r + 1][0].y : above.y) + 1.0f);
-                fy += ky[r][1] * (p[r][1].y - (r < RG_ROWS - 1 ? p[r + 1][1].y : above.w) + 1.0f);
+                qx += kx[r][0] * (p[r][0].x - p[r][1].x + 1.0f);
+                qx += kx[r][1] * (p[r][1].x - pr + 1.0f);
+                qy += ky[r][0] * (p[r][0].y - (r < RG_ROWS - 1 ? p[r + 1][0].y : above.y) + 1.0f);
+                qy += ky[r][1] * (p[r][1].y - (r < RG_ROWS - 1 ? p[r + 1][1].y : above.w) + 1.0f);
             }
-            double qx = fx, qy = fy;
             for (int off = span / 2; off > 0; off >>= 1) {
                 qx += __shfl_xor_sync(0xffffffffu, qx, off);
                 qy += __shfl_xor_sync(0xffffffffu, qy, off);
@@ -247,7 +343,7 @@ __global__ void __launch_bounds__(RG_THREADS, 1) darcy_group_kernel(const float 
                 }
             }
             if (mine && warp == q.w0 && q.row == 0 && q.col == 0)
-                cw[leaf] = make_float4((float)log(qx / (s * s)), 1.0f, (float)log(qy / (s * s)), 1.0f);
+                cw[leaf] = make_float4((float)log(ldexp(qx / (s * s), unit)), 1.0f, (float)log(ldexp(qy / (s * s), unit)), 1.0f);
         }
         // every warp of the group has read that the list is empty before a smaller group of the next class, which
         // some of them may already belong to, puts its leaves into the same words

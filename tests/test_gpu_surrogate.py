@@ -425,3 +425,19 @@ def test_darcy_base_does_not_depend_on_the_other_sides_of_the_batch(counts):
             ref[side == s] = _base_from_predict(sur, x[side == s], 3)[0]
         for _ in range(20):
             np.testing.assert_array_equal(_base_from_predict(sur, x, 3)[0], ref)
+
+
+@pytest.mark.parametrize("sigma,bound", [(1.0, 3e-5), (3.0, 3e-4)])
+@pytest.mark.parametrize("unit", [-46.0, -27.6, 0.0, 27.6, 41.0])
+def test_darcy_base_holds_at_any_scale_of_k(unit, sigma, bound):
+    """The Darcy base against 64-bit solves with K scaled by 1e-20 to 6e17: squares of residuals stay clear of FP32's
+    ends, and sums across threads carry more than FP32. 3e-5 is the bound of the tests above; at sigma 3 a leaf's
+    contrast of about e^18 lets FP32 pressures ten times as far off. The reference is solved at the leaf's own scale."""
+    lbm = _lbm()
+    leaves = [sigma * synth.gaussian_random_field(s, s, max(1.0, s / 8), seed=100 * s + i) - 4.0 + unit
+              for s, n in ((4, 20), (8, 20), (16, 20), (32, 12), (64, 12)) for i in range(n)]
+    x = _inputs(len(leaves), 0, leaves)
+    with lbm.Surrogate(1, 0) as sur:
+        c, _ = _base_from_predict(sur, x, 3)
+    ref = np.array([S.target_base(lk.astype(np.float32).astype(np.float64) - unit, 3) for lk in leaves])[:, [0, 2]] + unit
+    np.testing.assert_allclose(c, ref, rtol=0, atol=bound)
