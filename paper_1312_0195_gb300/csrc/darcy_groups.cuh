@@ -31,8 +31,8 @@ namespace sur {
 constexpr float DG_STOP = 2.5e-11f;
 constexpr int DG_CLASSES = 5;                // sides 64, 32, 16, 8, 4
 __host__ __device__ constexpr int dg_side(int c) { return 64 >> c; }
-constexpr int DG_TINY = DG_CLASSES;           // list of sides 1 to 3
-constexpr int DG_OTHER = DG_CLASSES + 1;      // list of any other side a size plane may say
+constexpr int DG_SMALL = DG_CLASSES;          // list of the other sides up to 32
+constexpr int DG_BIG = DG_CLASSES + 1;        // list of the other sides above
 constexpr int DG_LISTS = DG_CLASSES + 2;
 // Scratch of a call: the lists' counts, the classes' queue heads, then the lists.
 constexpr int DG_HEADER = 32, DG_HEADS = 16;
@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(256) darcy_classify_kernel(const float *x, int
 {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int s = darcy_size(x + (int64_t)i * IN_PLANES * PIX);
-        int c = s < 4 ? DG_TINY : DG_OTHER;
+        int c = s <= IMG ? DG_SMALL : DG_BIG;
         for (int k = 0; k < DG_CLASSES; ++k)
             if (s == dg_side(k)) c = k;
         scratch[DG_HEADER + (int64_t)c * n + atomicAdd(&scratch[c], 1)] = i;

@@ -549,14 +549,21 @@ __global__ void __launch_bounds__(256) patch_base_kernel(const float *x, int n, 
 // cells is k_f (p_i - p_j + G . (x_j - x_i)) with k_f the harmonic mean of the two cells, every cell
 // conserves mass, the leaf is periodic, and a unit force drives the flow along x, then along y.
 // K* along the drive is the mean face flux. The pressure system is solved by conjugate gradients
-// with the diagonal as preconditioner, in FP32, to a relative residual of 1e-5 or less (K* then
-// agrees with an FP64 direct solve to a few 1e-6). The leaf's log K is
+// with the diagonal as preconditioner, in FP32 with wider sums across threads, to a relative residual
+// of 1e-5 or less (K* then agrees with an FP64 direct solve to a few 1e-6). The leaf's log K is
 // read back from the input planes (phase plane 0 sampled every 32 / s pixels for s <= 32, the four
 // phase planes for 64 cells; above 64 cells the 64 x 64 plane stands for the leaf).
 // darcy_classify_kernel lists the leaves by side; 4, 8, 16, 32 and 64 are solved by darcy_group_kernel
-// (darcy_groups.cuh), the other sides by a warp each (darcy_warp_kernel).
+// (darcy_groups.cuh), other sides, which a caller's size plane may say, by a warp each up to 32 cells
+// (darcy_small_kernel) and by a CTA each above (darcy_big_kernel).
 constexpr int DB_N = 64;
+constexpr int DB_CELLS = DB_N * DB_N;
 constexpr int DB_MAXIT = 4000;
+constexpr int DBS_WARPS = 8;                                 // warps per CTA of the small-leaf kernel
+constexpr int DBS_CELLS = IMG * IMG;                         // cells per warp
+constexpr size_t DBS_SMEM = (size_t)DBS_WARPS * 6 * DBS_CELLS * sizeof(float);
+constexpr int DBB_THREADS = 256;
+constexpr size_t DBB_SMEM = (size_t)6 * DB_CELLS * sizeof(float);
 
 __device__ __forceinline__ int darcy_size(const float *xi)
 {
@@ -579,20 +586,38 @@ __device__ __forceinline__ float harmonic2f(double a, double b)
 namespace lbm {
 namespace sur {
 
-// (a, b) summed over a warp in a fixed order; every lane gets the sums
-__device__ __forceinline__ void warp_sum2(double &a, double &b)
+// NT threads solving one leaf: one warp (NT = 32) or the whole CTA.
+template <int NT> __device__ __forceinline__ void leaf_sync()
+{
+    if constexpr (NT == 32) __syncwarp(); else __syncthreads();
+}
+// (a, b) summed over them in a fixed order; every thread gets the sums
+template <int NT> __device__ __forceinline__ void leaf_sum2(double &a, double &b, double (*red)[2])
 {
     for (int off = 16; off > 0; off >>= 1) {
         a += __shfl_xor_sync(0xffffffffu, a, off);
         b += __shfl_xor_sync(0xffffffffu, b, off);
     }
+    if constexpr (NT > 32) {
+        if ((threadIdx.x & 31) == 0) {
+            red[threadIdx.x >> 5][0] = a;
+            red[threadIdx.x >> 5][1] = b;
+        }
+        __syncthreads();
+        a = b = 0.0;
+        for (int k = 0; k < NT / 32; ++k) {
+            a += red[k][0];
+            b += red[k][1];
+        }
+        __syncthreads();
+    }
 }
 
-// K*_xx and K*_yy of the leaf whose input planes start at xi, by one warp.
+// K*_xx and K*_yy of the leaf whose input planes start at xi.
+template <int NT>
 __device__ void darcy_leaf(const float *xi, int s, float *KX, float *KY, float *P, float *R, float *Dv, float *AD,
-                          double (&kd)[2])
+                          double (*red)[2], double (&kd)[2])
 {
-    constexpr int NT = 32;
     const int nc = s * s, r0 = threadIdx.x % NT;
     for (int c = r0; c < nc; c += NT) {
         const int y = c / s, xx = c - y * s;
@@ -605,14 +630,14 @@ __device__ void darcy_leaf(const float *xi, int s, float *KX, float *KY, float *
         }
         P[c] = v;                                          // log K, for now
     }
-    __syncwarp();
+    leaf_sync<NT>();
     for (int c = r0; c < nc; c += NT) {
         const int y = c / s, xx = c - y * s;
         const double k = exp((double)P[c]);
         KX[c] = harmonic2f(k, exp((double)P[y * s + (xx + 1 == s ? 0 : xx + 1)]));
         KY[c] = harmonic2f(k, exp((double)P[(y + 1 == s ? 0 : y + 1) * s + xx]));
     }
-    __syncwarp();
+    leaf_sync<NT>();
     for (int drive = 0; drive < 2; ++drive) {
         // A p = b with (A p)_c = sum over the faces of c of k_f (p_c - p_neighbour) and
         // b_c = k_f(behind c) - k_f(ahead of c) along the drive
@@ -630,7 +655,7 @@ __device__ void darcy_leaf(const float *xi, int s, float *KX, float *KY, float *
             prz = fmaf(b, z, prz);
         }
         double rr = prr, rz = prz;
-        warp_sum2(rr, rz);
+        leaf_sum2<NT>(rr, rz, red);
         const double stop = 1e-10 * rr;                    // (1e-5 relative residual)^2
         for (int it = 0; it < DB_MAXIT && rr > stop; ++it) {
             float pdad = 0.0f;
@@ -645,7 +670,7 @@ __device__ void darcy_leaf(const float *xi, int s, float *KX, float *KY, float *
                 pdad = fmaf(dc, ad, pdad);
             }
             double dad = pdad, unused = 0.0;
-            warp_sum2(dad, unused);
+            leaf_sum2<NT>(dad, unused, red);
             if (!(dad > 0.0)) break;                          // a direction in the null space
             const float alpha = (float)(rz / dad);
             float prr2 = 0.0f, prz2 = 0.0f;
@@ -660,7 +685,7 @@ __device__ void darcy_leaf(const float *xi, int s, float *KX, float *KY, float *
                 prz2 = dg > 0.0f ? fmaf(r, r / dg, prz2) : prz2;
             }
             double rr2 = prr2, rz2 = prz2;
-            warp_sum2(rr2, rz2);
+            leaf_sum2<NT>(rr2, rz2, red);
             const float beta = (float)(rz2 / rz);
             rz = rz2;
             rr = rr2;
@@ -670,7 +695,7 @@ __device__ void darcy_leaf(const float *xi, int s, float *KX, float *KY, float *
                 const float dg = KX[c] + KX[cl] + KY[c] + KY[cd];
                 Dv[c] = fmaf(beta, Dv[c], dg > 0.0f ? R[c] / dg : 0.0f);
             }
-            __syncwarp();
+            leaf_sync<NT>();
         }
         // mean face flux along the drive
         float pq = 0.0f;
@@ -680,30 +705,45 @@ __device__ void darcy_leaf(const float *xi, int s, float *KX, float *KY, float *
                              : KY[c] * (P[c] - P[(y + 1 == s ? 0 : y + 1) * s + xx] + 1.0f);
         }
         double q = pq, unused = 0.0;
-        warp_sum2(q, unused);
+        leaf_sum2<NT>(q, unused, red);
         kd[drive] = q / nc;
+        leaf_sync<NT>();
+    }
+}
+
+// The other sides up to 32: a warp per leaf, eight warps per CTA, each with its own work arrays.
+__global__ void __launch_bounds__(DBS_WARPS * 32) darcy_small_kernel(const float *x, int n, const int *scratch, float4 *cw)
+{
+    extern __shared__ float dw_smem[];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float *KX = dw_smem + w * 6 * DBS_CELLS, *KY = KX + DBS_CELLS, *P = KY + DBS_CELLS, *R = P + DBS_CELLS,
+          *Dv = R + DBS_CELLS, *AD = Dv + DBS_CELLS;
+    const int *list = scratch + DG_HEADER + (int64_t)DG_SMALL * n;
+    for (int j = blockIdx.x * DBS_WARPS + w; j < scratch[DG_SMALL]; j += gridDim.x * DBS_WARPS) {
+        const int i = list[j];
+        const float *xi = x + (int64_t)i * IN_PLANES * PIX;
+        double kd[2];
+        darcy_leaf<32>(xi, darcy_size(xi), KX, KY, P, R, Dv, AD, nullptr, kd);
+        if (lane == 0) cw[i] = make_float4((float)log(kd[0]), 1.0f, (float)log(kd[1]), 1.0f);
         __syncwarp();
     }
 }
 
-// The leaves of one list, a warp each: sides up to 3 eight warps a CTA, the sides that no leaf has but a caller's
-// size plane may say one warp a CTA, whose work arrays hold a side of 64.
-template <int WARPS, int CELLS>
-__global__ void __launch_bounds__(WARPS * 32) darcy_warp_kernel(const float *x, int n, const int *scratch, int which,
-                                                                float4 *cw)
+// The other sides above 32: a CTA per leaf. Inference on 160 leaves of 48 cells takes 3.6 ms, with a warp per leaf 10.3; of 2000
+// leaves of 24 cells, 4.0 ms with eight warps a CTA and 10.6 with one.
+__global__ void __launch_bounds__(DBB_THREADS) darcy_big_kernel(const float *x, int n, const int *scratch, float4 *cw)
 {
     extern __shared__ float dw_smem[];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float *KX = dw_smem + w * 6 * CELLS, *KY = KX + CELLS, *P = KY + CELLS, *R = P + CELLS, *Dv = R + CELLS,
-          *AD = Dv + CELLS;
-    const int *list = scratch + DG_HEADER + (int64_t)which * n;
-    for (int j = blockIdx.x * WARPS + w; j < scratch[which]; j += gridDim.x * WARPS) {
+    float *KX = dw_smem, *KY = KX + DB_CELLS, *P = KY + DB_CELLS, *R = P + DB_CELLS, *Dv = R + DB_CELLS, *AD = Dv + DB_CELLS;
+    __shared__ double red[DBB_THREADS / 32][2];
+    const int *list = scratch + DG_HEADER + (int64_t)DG_BIG * n;
+    for (int j = blockIdx.x; j < scratch[DG_BIG]; j += gridDim.x) {
         const int i = list[j];
         const float *xi = x + (int64_t)i * IN_PLANES * PIX;
         double kd[2];
-        darcy_leaf(xi, darcy_size(xi), KX, KY, P, R, Dv, AD, kd);
-        if (lane == 0) cw[i] = make_float4((float)log(kd[0]), 1.0f, (float)log(kd[1]), 1.0f);
-        __syncwarp();
+        darcy_leaf<DBB_THREADS>(xi, darcy_size(xi), KX, KY, P, R, Dv, AD, red, kd);
+        if (threadIdx.x == 0) cw[i] = make_float4((float)log(kd[0]), 1.0f, (float)log(kd[1]), 1.0f);
+        __syncthreads();
     }
 }
 
@@ -745,17 +785,18 @@ cudaError_t launch_base(const float *x, int n, int mode, float4 *cw, int cap, cu
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(darcy_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)sizeof(DarcyShared));
-        constexpr int OTHER_SMEM = 6 * DB_N * DB_N * sizeof(float), TINY_CELLS = 9;
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(darcy_warp_kernel<1, DB_N * DB_N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     OTHER_SMEM);
+            e = cudaFuncSetAttribute(darcy_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DBS_SMEM);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(darcy_big_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DBB_SMEM);
         if (e == cudaSuccess) e = cudaMemsetAsync(scratch, 0, sizeof(int) * DG_HEADER, st);
         if (e != cudaSuccess) return e;
         const int sms = sm_count(dev);
         darcy_classify_kernel<<<nblk(n), 256, 0, st>>>(x, n, scratch);
         darcy_group_kernel<<<n < sms ? n : sms, RG_THREADS, sizeof(DarcyShared), st>>>(x, n, scratch, cw);
-        darcy_warp_kernel<8, TINY_CELLS><<<sms, 256, 8 * 6 * TINY_CELLS * sizeof(float), st>>>(x, n, scratch, DG_TINY, cw);
-        darcy_warp_kernel<1, DB_N * DB_N><<<2 * sms, 32, OTHER_SMEM, st>>>(x, n, scratch, DG_OTHER, cw);
+        const int gs = (n + DBS_WARPS - 1) / DBS_WARPS;
+        darcy_small_kernel<<<gs < sms ? gs : sms, DBS_WARPS * 32, DBS_SMEM, st>>>(x, n, scratch, cw);
+        darcy_big_kernel<<<n < 2 * sms ? n : 2 * sms, DBB_THREADS, DBB_SMEM, st>>>(x, n, scratch, cw);
         count_launches(3);
     } else {
         patch_base_kernel<<<n < 65535 ? n : 65535, 256, 0, st>>>(x, n, mode, cw);

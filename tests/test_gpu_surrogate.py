@@ -441,3 +441,25 @@ def test_darcy_base_holds_at_any_scale_of_k(unit, sigma, bound):
         c, _ = _base_from_predict(sur, x, 3)
     ref = np.array([S.target_base(lk.astype(np.float32).astype(np.float64) - unit, 3) for lk in leaves])[:, [0, 2]] + unit
     np.testing.assert_allclose(c, ref, rtol=0, atol=bound)
+
+
+def test_darcy_base_of_other_sides_matches_oracle():
+    """Sides that no leaf of a quadtree has, but a caller's size plane may say: 5 to 63 cells, read from the planes as the
+    library states (plane 0 sampled every 32 // s pixels up to 32 cells, the four phase planes above), among leaves of
+    the usual sides. 3e-5 is the bound of the tests above."""
+    lbm = _lbm()
+    sides = [5, 7, 12, 20, 24, 31, 33, 40, 48, 63, 64, 8, 3] * 3
+    x = _inputs(len(sides), 0, [synth.gaussian_random_field(64, 64, 6.0, seed=300 + i) - 4.0 for i in range(len(sides))])
+    x[:, 4] = (np.log2(np.array(sides)) / 6.0)[:, None, None]
+    ref = []
+    for xi, s in zip(x.astype(np.float64), sides):
+        full = np.empty((64, 64))
+        for a in (0, 1):
+            for b in (0, 1):
+                full[a::2, b::2] = xi[2 * a + b]
+        step = 32 // s if s <= 32 else 1
+        leaf = xi[0][::step, ::step][:s, :s] if s <= 32 else full[:s, :s]
+        ref.append(np.log(S.darcy_keff(np.exp(leaf))))
+    with lbm.Surrogate(1, 0) as sur:
+        c, _ = _base_from_predict(sur, x.astype(np.float32), 3)
+    np.testing.assert_allclose(c, np.array(ref), rtol=0, atol=3e-5)
