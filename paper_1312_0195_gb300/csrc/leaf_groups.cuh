@@ -41,7 +41,7 @@ struct RegGeo {
     int scratch;                 // first of this lane's leaf's cells in an array of the CTA's 4096
 };
 
-__device__ __forceinline__ RegGeo reg_geometry(int s, int warp, int lane)
+__host__ __device__ __forceinline__ RegGeo reg_geometry(int s, int warp, int lane)
 {
     RegGeo q;
     const int w = s / 2, per_warp = 32 / w, blocks = s / RG_ROWS;

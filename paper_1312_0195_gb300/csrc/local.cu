@@ -945,6 +945,8 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) local_keff_kernel(LocalArgs 
             fresh = __syncthreads_or(tid < nslots && (hot[tid].z & 4)) != 0;
         }
     }
+    // started beside the register solver (launch_solvers): whoever waits for this kernel waits for that one too
+    if (tid == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 using LocalKernel = void (*)(LocalArgs);
@@ -1092,20 +1094,45 @@ __global__ void __launch_bounds__(256) abandon_kernel(LocalArgs a, int reg_block
     }
 }
 
-// Launches the solvers of a batch on `blocks` CTAs: from rest in FP32, sides that are multiples of 4
+// Launches the solvers of a batch on at most `sms` CTAs each: from rest in FP32, sides that are multiples of 4
 // go to the register solver (1.2 to 2.3 times the rate of the shared-memory one at every such side, see
 // local_reg.cuh) and the rest to the shared-memory one; everything else to the latter.
 // reg, other: whether the batch has sides of either kind (both, if only the device knows).
-cudaError_t launch_solvers(LocalArgs &a, bool f64, double tau, bool lg, int blocks, bool reg, bool other,
+//
+// A batch of both kinds runs both solvers side by side: the second launch may start once every CTA of the first has
+// (griddepcontrol), needs nothing of it, and waits for it before it ends. Either takes a whole SM for a CTA. The first
+// gets the SMs that the second's jobs leave free, and at least a share by the CTAs that hold each side's jobs at once
+// and their time for a step (1.3 and 2.2 us), so that short lists of either do not wait; CTAs of the second take
+// over SMs that the first gives back.
+// Milliseconds in the shared-memory solver alone / one launch after the other / side by side:
+// one leaf of every side from 1 to 40, 2000 steps 3.6 / 6.0 / 3.7, to the tolerance 34 / 52 / 35; fifty of each, 1000
+// steps 9.7 / 10.5 / 9.9; twenty of each, to the tolerance 82 / 131 / 84; 4000 leaves of 16 cells and 40 of 15, to the
+// tolerance 47 / 37 / 22, 40 and 4000 43 / 51 / 44. With SMs by cells alone, twenty of each took 99.
+cudaError_t launch_solvers(LocalArgs &a, bool f64, double tau, bool lg, int sms, bool reg, bool other,
                            cudaStream_t st)
 {
     const bool use_reg = !f64 && !lg && !a.warm;
-    if (use_reg && reg) {
+    int reg_blocks = use_reg && reg ? sms : 0, blocks = sms;
+    if (!a.table) {                                               // jobs are known here
+        double jobs[2] = {0.0, 0.0}, hold[2] = {0.0, 0.0};        // of the shared-memory solver, of the register solver
+        for (int c = 0; c < a.nclass; ++c) {
+            const int s = a.class_size[c], n = a.class_off[c + 1] - a.class_off[c], r = use_reg && reg_side(s);
+            const RegGeo q = reg_geometry(r ? s : 4, 0, 0);
+            jobs[r] += n;
+            hold[r] += (double)n / (r ? RG_WARPS / q.group * q.jobs : std::min(LocalCfg<float>::CMAX / (s * s), MAXSLOTS));
+        }
+        const double few = sms / 8;
+        double share = std::max(sms * 1.3 * hold[1] / (1.3 * hold[1] + 2.2 * hold[0]), std::min(std::ceil(hold[1]), few));
+        share = std::max(std::min(share, sms - std::min(std::ceil(hold[0]), few)), sms - jobs[0]);
+        reg_blocks = std::min(reg_blocks, std::max(1, (int)std::min(share, jobs[1])));
+        blocks = std::min(sms, std::max(1, (int)std::min(jobs[0], 1e6)));
+    }
+    if (reg_blocks > 0) {
         const auto kern = tau == 1.0 ? local_reg_kernel<true> : local_reg_kernel<false>;
         const cudaError_t e =
             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RegShared));
         if (e != cudaSuccess) return e;
-        kern<<<blocks, RG_THREADS, sizeof(RegShared), st>>>(a);
+        kern<<<reg_blocks, RG_THREADS, sizeof(RegShared), st>>>(a);
         count_launches(1);
     }
     if (!use_reg || other) {
@@ -1113,12 +1140,23 @@ cudaError_t launch_solvers(LocalArgs &a, bool f64, double tau, bool lg, int bloc
         const LocalKernel kern = lg ? local_kernel_lg(f64, tau) : local_kernel(f64, tau, a.warm);
         const size_t smem = lg ? (f64 ? lg_smem<double>() : lg_smem<float>())
                                : f64 ? LocalCfg<double>::SMEM : LocalCfg<float>::SMEM;
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        kern<<<blocks, LOCAL_THREADS, smem, st>>>(a);
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.gridDim = dim3((unsigned)blocks);
+        cfg.blockDim = dim3(LOCAL_THREADS);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cfg.attrs = attr;
+        cfg.numAttrs = reg_blocks > 0 ? 1 : 0;
+        e = cudaLaunchKernelEx(&cfg, kern, a);
+        if (e != cudaSuccess) return e;
         count_launches(1);
     }
-    abandon_kernel<<<1, 256, 0, st>>>(a, use_reg && reg ? blocks : 0);
+    abandon_kernel<<<1, 256, 0, st>>>(a, reg_blocks);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -1283,10 +1321,7 @@ lbm_status local_keff_core(const lbm_params *p, const float *kappa_dev, const lb
         }
         a.class_off[a.nclass] = off[a.nclass];
         a.heads = d_heads;
-        int blocks = sm_count(dev);
-        const int64_t max_useful = (int64_t)jobs.size();
-        if (blocks > max_useful) blocks = (int)max_useful;
-        LOC_CUDA2(launch_solvers(a, f64, p->tau, lg != nullptr, blocks, reg, other, st));
+        LOC_CUDA2(launch_solvers(a, f64, p->tau, lg != nullptr, sm_count(dev), reg, other, st));
     } else {
         a.nclass = 1;
         for (int i = 0; i < n_leaves; ++i) {
@@ -1712,9 +1747,7 @@ extern "C" lbm_status lbm_local_keff_batch_noalloc(const lbm_params *p, const fl
     a.time_limit_ns = (unsigned long long)(g_time_limit_s * 1e9);
     bool reg = false, other = false;
     for (int c = 0; c < a.nclass; ++c) (reg_side(a.class_size[c]) ? reg : other) = true;
-    int blocks = sm_count(dev);
-    if (blocks > 2 * n_leaves) blocks = 2 * n_leaves;
-    NA_CUDA(launch_solvers(a, f64, p->tau, false, blocks, reg, other, st));
+    NA_CUDA(launch_solvers(a, f64, p->tau, false, sm_count(dev), reg, other, st));
     int flags[2] = {0, 0};
     NA_CUDA(cudaMemcpyAsync(flags, scr + NA_FLAGS + 1, sizeof flags, cudaMemcpyDeviceToHost, st));
     NA_CUDA(cudaStreamSynchronize(st));

@@ -241,7 +241,10 @@ __global__ void __launch_bounds__(RG_THREADS, 1) local_reg_kernel(LocalArgs a)
     extern __shared__ __align__(16) unsigned char rg_smem[];
     RegShared &sh = *reinterpret_cast<RegShared *>(rg_smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) sh.t0 = globaltimer();
+    if (tid == 0) {
+        sh.t0 = globaltimer();
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the shared-memory solver needs nothing of this one
+    }
     if (lane == 0) sh.abort[warp] = 0;
     __syncthreads();
     const int nclass = a.table ? (a.table[DT_BAD] ? 0 : a.table[DT_NCLASS]) : a.nclass;

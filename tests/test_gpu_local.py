@@ -371,3 +371,29 @@ def test_time_limit_reaches_jobs_still_in_the_queue(storage, warm):
         assert torch.isnan(ke.reshape(-1, 2, 2)[:, 0, :][steps == 0]).all()
     finally:
         lbm.lbm_set_time_limit(600.0)
+
+
+@pytest.mark.parametrize("sizes,steps,tol", [(range(1, 41), 300, 0.0), ([16] * 40 + [15] * 900, 200000, 1e-6),
+                                             ([64] * 3 + [12] * 500 + [63, 2], 200000, 1e-6)])
+def test_batches_of_both_solvers_equal_their_halves(sizes, steps, tol):
+    """A batch whose sides go to both solvers runs them side by side; K*, status and steps of a leaf are those of a batch of
+    its own kind bit for bit, and the outputs are complete when the call returns (read at once, ten times over)."""
+    import torch
+    lbm = _lbm()
+    kap = torch.from_numpy(synth.lognormal_kappa(512, 512, 8.0, 1.0, seed=27).astype(np.float32)).cuda()
+    r = np.random.default_rng(5)
+    size = r.permutation(np.array(list(sizes)))
+    leaves = np.stack([r.integers(0, 513 - size), r.integers(0, 513 - size), size], axis=1).astype(np.int32)
+    p = lbm.Params(nx=512, ny=512, tau=1.0)
+
+    def run(lv):
+        return [t.cpu() for t in lbm.local_keff(p, kap, torch.from_numpy(lv).cuda(), 1e-6, tol, steps, 64)[:3]]
+
+    reg = (size >= 4) & (size % 4 == 0)
+    ref = [torch.empty((len(leaves), *t.shape[1:]), dtype=t.dtype) for t in run(leaves[:1])]
+    for which in (reg, ~reg):
+        for a, b in zip(ref, run(leaves[which])):
+            a[torch.from_numpy(which)] = b
+    for _ in range(10):
+        for a, b in zip(run(leaves), ref):
+            assert torch.equal(a, b)
