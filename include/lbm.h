@@ -290,8 +290,9 @@ lbm_status lbm_local_keff_lg(const lbm_params *p, const float *kappa_dev, int32_
                              const double *keff_fallback_dev, double *keff_dev, int32_t *status_dev,
                              int32_t *steps_dev, double *window_dev, int32_t *n_fallback, void *cuda_stream);
 
-/* Wall-clock bound (seconds, > 0) of one local-problem launch; past it the
- * kernel abandons its remaining jobs with LBM_ETIMEOUT instead of running on.
+/* Wall-clock bound (seconds, > 0) of a batch of local problems, from its first
+ * launch on (per leaf with persistent = 0); past it the kernels abandon the
+ * remaining jobs with LBM_ETIMEOUT instead of running on.
  * Process-wide; default 600 s. */
 lbm_status lbm_set_time_limit(double seconds);
 

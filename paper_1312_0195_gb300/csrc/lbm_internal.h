@@ -166,6 +166,7 @@ enum DeviceTable {
     DT_WORST = 325,           // worst per-leaf status of the solver
     DT_ABORT = 326,           // the solver's wall-clock limit ran out
     DT_NFALLBACK = 327,       // leaves sent to the solver
+    DT_START = 328,           // [2] start of the wall-clock limit (64 bits)
     DT_INTS = 384
 };
 

@@ -94,6 +94,7 @@ struct LocalArgs {
     int *worst;               // [1] (zeroed)
     int *abort_flag;          // [1] (zeroed)
     unsigned long long time_limit_ns;
+    unsigned long long *t_start;   // [1] when the call's first CTA started (zeroed), or nullptr: each launch its own
     int skip_reg;             // 1: sides of the register solver (local_reg.cuh) are not taken here
 };
 
@@ -109,6 +110,13 @@ __device__ __forceinline__ unsigned long long globaltimer()
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
+}
+
+// the start of the wall-clock limit, the same for every CTA of a call's launches
+__device__ __forceinline__ unsigned long long start_time(const LocalArgs &a)
+{
+    const unsigned long long now = globaltimer(), first = a.t_start ? atomicCAS(a.t_start, 0ull, now) : 0ull;
+    return first ? first : now;
 }
 
 // drag fraction e = 1 - d = eps nu / (2 kappa + eps nu) of Eq. 6 (see the fine-grid step)
@@ -668,7 +676,7 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) local_keff_kernel(LocalArgs 
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const T hg = kc<T>(a, K_HG);
     if (tid == 0) {
-        s_t0 = globaltimer();
+        s_t0 = start_time(a);
         s_abort = 0;
         // this solver's classes (a table is built on the device by an earlier kernel of the same stream). Skipping the
         // others here and not in the loop keeps a branch out of it that slowed every step by 3 %.
@@ -1294,15 +1302,16 @@ lbm_status local_keff_core(const lbm_params *p, const float *kappa_dev, const lb
     } while (0)
     LOC_CUDA2(cudaMalloc(&d_jobs, sizeof(int) * jobs.size()));
     LOC_CUDA2(cudaMalloc(&d_heads, sizeof(int) * nheads));
-    LOC_CUDA2(cudaMalloc(&d_flags, sizeof(int) * 2));
+    LOC_CUDA2(cudaMalloc(&d_flags, sizeof(int) * 4));             // worst status, abort flag, start (64 bits)
     LOC_CUDA2(cudaMemcpyAsync(d_jobs, jobs.data(), sizeof(int) * jobs.size(), cudaMemcpyHostToDevice, st));
     LOC_CUDA2(cudaMemsetAsync(d_heads, 0, sizeof(int) * nheads, st));
-    LOC_CUDA2(cudaMemsetAsync(d_flags, 0, sizeof(int) * 2, st));
+    LOC_CUDA2(cudaMemsetAsync(d_flags, 0, sizeof(int) * 4, st));
     LOC_CUDA2(cudaMemsetAsync(status_dev, 0, sizeof(int32_t) * n_leaves, st));
     if (steps_dev) LOC_CUDA2(cudaMemsetAsync(steps_dev, 0, sizeof(int32_t) * 2 * n_leaves, st));
     a.jobs = d_jobs;
     a.worst = d_flags;
     a.abort_flag = d_flags + 1;
+    if (persistent) a.t_start = reinterpret_cast<unsigned long long *>(d_flags + 2);
 
     const bool f64 = p->storage == LBM_F64;
     int dev = 0;
@@ -1496,6 +1505,7 @@ lbm_status launch_local_from_table(const lbm_params *p, const float *kappa_dev, 
     a.steps = steps_dev;
     a.worst = table + DT_WORST;
     a.abort_flag = table + DT_ABORT;
+    a.t_start = reinterpret_cast<unsigned long long *>(table + DT_START);
     a.time_limit_ns = (unsigned long long)(time_limit_s * 1e9);
     // one CTA per SM; CTAs of an empty table find no class and return at once
     int dev = 0;
@@ -1578,7 +1588,8 @@ constexpr int NA_CURSOR = 65;                 // [65] scatter cursors per size
 constexpr int NA_HEADS = 130;                 // [64] queue heads per class
 constexpr int NA_FLAGS = 194;                 // [4]  bad-leaf flag, worst status, abort flag, spare
 constexpr int NA_TABLE = 198;                 // [1 + 64 + 65] nclass, class_size[], class_off[]
-constexpr int NA_HEADER = 328;                // ints before the job list (keeps it 32-byte aligned)
+constexpr int NA_START = 328;                 // [2] start of the wall-clock limit
+constexpr int NA_HEADER = 336;                // ints before the job list (keeps it 32-byte aligned)
 constexpr int NA_JOBS = NA_HEADER;            // [2 * NOALLOC_MAX_LEAVES]
 constexpr int NA_TOTAL = NA_JOBS + 2 * NOALLOC_MAX_LEAVES;
 
@@ -1740,6 +1751,7 @@ extern "C" lbm_status lbm_local_keff_batch_noalloc(const lbm_params *p, const fl
     a.steps = steps_dev;
     a.worst = scr + NA_FLAGS + 1;
     a.abort_flag = scr + NA_FLAGS + 2;
+    a.t_start = reinterpret_cast<unsigned long long *>(scr + NA_START);
     a.time_limit_ns = (unsigned long long)(g_time_limit_s * 1e9);
     bool reg = false, other = false;
     for (int c = 0; c < a.nclass; ++c) (reg_side(a.class_size[c]) ? reg : other) = true;

@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(RG_THREADS, 1) local_reg_kernel(LocalArgs a)
     RegShared &sh = *reinterpret_cast<RegShared *>(rg_smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
-        sh.t0 = globaltimer();
+        sh.t0 = start_time(a);
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the shared-memory solver needs nothing of this one
     }
     if (lane == 0) sh.abort[warp] = 0;

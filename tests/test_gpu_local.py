@@ -397,3 +397,40 @@ def test_batches_of_both_solvers_equal_their_halves(sizes, steps, tol):
     for _ in range(10):
         for a, b in zip(run(leaves), ref):
             assert torch.equal(a, b)
+
+
+def test_time_limit_covers_both_solvers_of_a_batch():
+    """The limit counts from the batch's first launch. With a queue built on the device the register solver takes every
+    SM, and the shared-memory solver its jobs after it: a limit that either would meet alone, but not both, runs out.
+    Leaves of 16 and 1 cells with a margin of 2 are patches of 20 (register solver) and 5 (shared-memory solver)."""
+    import time
+
+    import torch
+    lbm = _lbm()
+    kap = torch.from_numpy(synth.lognormal_kappa(512, 512, 8.0, 1.0, seed=29).astype(np.float32)).cuda()
+    r = np.random.default_rng(6)
+    p = lbm.Params(nx=512, ny=512, tau=1.0, margin=2)
+
+    def leaves(s, n):
+        return np.stack([r.integers(0, 513 - s, n), r.integers(0, 513 - s, n), np.full(n, s)], axis=1).astype(np.int32)
+
+    reg, other = leaves(16, 4000), leaves(1, 16000)
+    with lbm.Surrogate(2, 0) as sur:
+        def run(lv):
+            lv = torch.from_numpy(lv).cuda()
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            st, nfb, worst = sur.keff(p, kap, lv, 1e-30, 1e-6, 0.0, 60000)[2:]
+            return time.perf_counter() - t0, nfb, worst, st.cpu().numpy()
+
+        run(reg[:10])
+        t = [run(reg), run(other)]
+        limit = 1.3 * max(t[0][0], t[1][0])
+        assert [x[1:3] for x in t] == [(len(reg), lbm.LBM_OK), (len(other), lbm.LBM_OK)]
+        assert t[0][0] + t[1][0] > 1.2 * limit, t
+        try:
+            lbm.lbm_set_time_limit(limit)
+            both = run(np.concatenate([reg, other]))
+            assert both[2] == lbm.LBM_ETIMEOUT and (both[3][:len(reg)] == lbm.LBM_OK).all()
+        finally:
+            lbm.lbm_set_time_limit(600.0)
