@@ -134,7 +134,10 @@ lbm_status lbm_grid_destroy(lbm_grid *g);
  * is computed in FP64; when tol_rel > 0 and r <= tol_rel the call stops and
  * returns LBM_OK. tol_rel <= 0 runs exactly max_steps and returns LBM_OK.
  * If tol_rel > 0 and the test never passes, returns LBM_ENOTCONV (the state is
- * valid). steps_done (may be NULL) receives the steps taken by this call;
+ * valid). LBM_ETIMEOUT: a wait between the blocks that step a small lattice
+ * exceeded the limit of lbm_set_time_limit; the grid then holds no valid state,
+ * and its calls return LBM_ETIMEOUT until lbm_grid_load_state.
+ * steps_done (may be NULL) receives the steps taken by this call;
  * residual (may be NULL) the last residual computed in this call, or -1. */
 lbm_status lbm_step(lbm_grid *g, int64_t max_steps, double tol_rel, int32_t check_every,
                     int64_t *steps_done, double *residual);
@@ -292,7 +295,8 @@ lbm_status lbm_local_keff_lg(const lbm_params *p, const float *kappa_dev, int32_
 
 /* Wall-clock bound (seconds, > 0) of a batch of local problems, from its first
  * launch on (per leaf with persistent = 0); past it the kernels abandon the
- * remaining jobs with LBM_ETIMEOUT instead of running on.
+ * remaining jobs with LBM_ETIMEOUT instead of running on. Also the bound of
+ * the waits between the blocks of a small lattice's step (lbm_step).
  * Process-wide; default 600 s. */
 lbm_status lbm_set_time_limit(double seconds);
 

@@ -25,7 +25,6 @@ lbm_status local_keff_impl(const lbm_params *p, const float *kappa_dev, const lb
                            double g_const, double tol_rel, int64_t max_steps, int32_t check_every,
                            int32_t persistent, double *keff_dev, int32_t *status_dev, int32_t *steps_dev,
                            void *cuda_stream, double time_limit_s);
-double local_time_limit();
 lbm_status upscale_with_surrogate(const lbm_params *p, const float *kappa_dev, int32_t block, lbm_surrogate *s,
                                   double spread_max, double g_const, double tol_rel, int64_t max_steps,
                                   double *keff_dev, int32_t *n_fallback, void *cuda_stream);

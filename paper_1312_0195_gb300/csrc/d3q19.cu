@@ -26,7 +26,6 @@ namespace lbm {
 lbm_status fail(lbm_status s, const char *fmt, ...);
 bool is_device_ptr(const void *p);
 void count_launches(int64_t n);
-double local_time_limit();
 
 namespace {
 

@@ -142,6 +142,7 @@ struct lbm_grid {
     GridLaunch L{};
     int64_t t = 0;
     int sms = 1;
+    bool lost = false;               // a step gave up halfway: no valid state until one is loaded
     bool fused = false;              // several steps per pass (multistep.cu) where a call takes several
     TileGeom tiles{0, 0, 0, 0, 0};   // ntx > 0: a small lattice, stepped in shared memory (tiles.cu)
     void *mem = nullptr;             // the one allocation behind every device pointer of the grid
@@ -247,7 +248,8 @@ static cudaError_t enqueue_multi(const lbm_grid *g, int src_idx, int nlev, unsig
 // outcome's bits.
 static cudaError_t enqueue_tiles(lbm_grid *g, int n, int check_every, int *checks)
 {
-    TileRun run{n, 0, check_every, g->tile_result, g->tile_exch, g->tile_base, &g->outcome->tile_err};
+    TileRun run{n, 0, check_every, g->tile_result, g->tile_exch, g->tile_base, &g->outcome->tile_err,
+                (int)std::min(TILE_POLLS * local_time_limit(), 2e9)};
     *checks = 0;
     if (check_every > 0) {
         run.first_check = (int)(check_every - g->t % check_every);
@@ -274,6 +276,13 @@ static cudaError_t enqueue_tiles(lbm_grid *g, int n, int check_every, int *check
     g->tile_base += n / TILE_HALO + 1;
     g->cur = 1 - g->cur;
     return e;
+}
+
+// LBM_OK, unless the grid holds no valid state.
+static lbm_status valid_state(const lbm_grid *g)
+{
+    if (!g->lost) return LBM_OK;
+    return fail(LBM_ETIMEOUT, "an earlier step of this grid gave up halfway: load a state before going on");
 }
 
 // The outcome of the calls so far, after a synchronisation with the grid's stream.
@@ -661,6 +670,8 @@ lbm_status lbm_step(lbm_grid *g, int64_t max_steps, double tol_rel, int32_t chec
     if (check_every < 0) return fail(LBM_EINVAL, "check_every must be >= 0");
     if (!std::isfinite(tol_rel)) return fail(LBM_EINVAL, "tol_rel must be finite");
     if (tol_rel > 0.0 && check_every == 0) return fail(LBM_EINVAL, "tol_rel > 0 needs check_every > 0");
+    const lbm_status valid = valid_state(g);
+    if (valid != LBM_OK) return valid;
     DeviceGuard dg(g->dev);
     if (tol_rel > 0.0 && !g->h_outcome) LBM_CUDA(cudaMallocHost(&g->h_outcome, sizeof *g->h_outcome));
     const int CHUNK = 1024;
@@ -738,9 +749,11 @@ lbm_status lbm_step(lbm_grid *g, int64_t max_steps, double tol_rel, int32_t chec
     } else {
         LBM_CUDA(cudaStreamSynchronize(g->stream));
     }
-    if (o.tile_err) {                                        // the state is not valid any more
-        cudaMemsetAsync(&g->outcome->tile_err, 0, sizeof(int), g->stream);
-        return fail(LBM_ECUDA, "a wait between the tiles of the lattice gave up");
+    if (o.tile_err) {
+        g->lost = true;
+        LBM_CUDA(cudaMemsetAsync(&g->outcome->tile_err, 0, sizeof(int), g->stream));
+        return fail(LBM_ETIMEOUT, "a wait between the tiles of the lattice exceeded %.3g s: the state is not valid any more",
+                    local_time_limit());
     }
     if (checked && tol_rel <= 0.0) resid = residual_of(o, as_bits);
     if (steps_done) *steps_done = done;
@@ -756,6 +769,8 @@ lbm_status lbm_get_fields(lbm_grid *g, float *rho_dev, float *u_dev, float *v_de
     if (!g) return fail(LBM_EINVAL, "grid is NULL");
     if ((rho_dev && !is_device_ptr(rho_dev)) || (u_dev && !is_device_ptr(u_dev)) || (v_dev && !is_device_ptr(v_dev)))
         return fail(LBM_EINVAL, "field outputs must be device pointers");
+    const lbm_status valid = valid_state(g);
+    if (valid != LBM_OK) return valid;
     DeviceGuard dg(g->dev);
     LBM_CUDA(enqueue_moments(g, g->cur, -1, rho_dev, u_dev, v_dev, g->stream));
     count_launches(1);
@@ -766,6 +781,8 @@ lbm_status lbm_get_fields(lbm_grid *g, float *rho_dev, float *u_dev, float *v_de
 lbm_status lbm_mean_velocity(lbm_grid *g, double out_mean_uv[2])
 {
     if (!g || !out_mean_uv) return fail(LBM_EINVAL, "grid or output is NULL");
+    const lbm_status valid = valid_state(g);
+    if (valid != LBM_OK) return valid;
     DeviceGuard dg(g->dev);
     LBM_CUDA(enqueue_moments(g, g->cur, -1, nullptr, nullptr, nullptr, g->stream));
     LBM_CUDA(launch_reduce_partials(g->partials, g->L.mom_blocks, g->outcome->sums, g->stream));
@@ -819,6 +836,8 @@ lbm_status lbm_grid_save_state(lbm_grid *g, void *state_dev, int64_t nbytes, int
         return fail(LBM_EINVAL, "state buffer holds %lld bytes, the grid's state is %lld", (long long)nbytes,
                     (long long)lbm_grid_state_bytes(g));
     if (!is_device_ptr(state_dev)) return fail(LBM_EINVAL, "state_dev is not a device pointer");
+    const lbm_status valid = valid_state(g);
+    if (valid != LBM_OK) return valid;
     DeviceGuard dg(g->dev);
     const size_t half = 9 * g->plane * storage_bytes(g->p.storage);
     const CkptHeader h = grid_header(g);
@@ -855,6 +874,7 @@ lbm_status lbm_grid_load_state(lbm_grid *g, const void *state_dev, int64_t nbyte
     LBM_CUDA(cudaMemcpyAsync(g->buf[1 - g->cur], src + CKPT_HEADER_BYTES + half, half, cudaMemcpyDeviceToDevice,
                              g->stream));
     LBM_CUDA(cudaStreamSynchronize(g->stream));
+    g->lost = false;
     g->t = steps;
     return LBM_OK;
 }

@@ -95,21 +95,26 @@ TileGeom tile_geometry(int storage, int coef_mode, bool gfield, int nx, int ny, 
 // back and reading the outcome cost about 20 us. Microseconds of a call here / in passes of four: 12 steps 31 / 33 at
 // 128 x 64, 46 / 47 at 517 x 389, 52 / 44 at 500 x 500, the largest; 16 steps 60 / 55 and 24 steps 77 / 76 there.
 constexpr int TILES_FROM = 16;
+constexpr double TILE_POLLS = 2.1e6;    // polls of a thread in a second at most: a round trip to L2 each
 constexpr size_t tile_exchange_bytes(int64_t cells) { return (size_t)cells * 2 * 3 * 16; }
 // One launch: `steps` steps from the state in src, with the residual's maxima (bits of max |du| and max |u|) after
 // step first_check and every check_every-th step on (check_every = 0: none) raised in result[2 c], result[2 c + 1] for
 // the c-th of them (zeroed before). dst gets the newest state, src the one before it. exch: the exchanges' words,
 // tile_exchange_bytes, zeroed once; base: the number of exchanges that have gone through it; err: set if a wait
-// between CTAs gave up.
+// between CTAs gave up, after `patience` polls of a thread in
+// one exchange.
 struct TileRun {
     int steps, first_check, check_every;
     unsigned *result;
     void *exch;
     unsigned base;
     int *err;
+    int patience;
 };
 cudaError_t launch_tiles(int storage, int coef_mode, bool gfield, bool walls, const void *args, const TileGeom &g,
                          const TileRun &run, cudaStream_t st);
+
+double local_time_limit();   // seconds, lbm_set_time_limit (local.cu)
 
 // ---- launch counter (lbm_api.cu) ----------------------------------------------
 void count_launches(int64_t n);

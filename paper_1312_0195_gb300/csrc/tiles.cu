@@ -5,7 +5,10 @@
 // tiles per SM, each with a halo of four cells. A CTA keeps two tiles in shared memory, interleaved cell
 // by cell (the two tiles' values are the lanes of packed f32x2 operands), steps them four times while the halo is
 // used up from outside in, and then exchanges its tiles' outer four rings for its halo through global memory (L2).
-// The launch is cooperative, so all CTAs are resident while they wait for one another; every wait is bounded.
+// The launch is cooperative, so all CTAs become resident, and wait for one another in bounded time: a thread gives up
+// after as many polls in vain as the limit of lbm_set_time_limit has room for, which is long enough for other
+// streams' kernels to leave the SMs that some CTAs may still have to wait for. (Reading a clock at each such poll
+// made the coarse run of 256 x 256 2 % slower.)
 // Two areas take the exchanges in turn: an area is written again two exchanges later, when words of the exchange
 // between have come in from every CTA that read it.
 // Every cell's arithmetic is that of the one-step kernel, so the bits are the same.
@@ -26,7 +29,6 @@ namespace {
 constexpr int TL_THREADS = 768;
 constexpr int TL_ROUNDS = 2;                         // cells of a thread at most
 constexpr int TL_ITEMS = 3;                          // halo cells (and outer-ring cells) of a thread at most
-constexpr int TL_SPINS = 1 << 21;                    // polls of a flag before a wait gives up (about a second)
 
 // Cells of a tile with its halo that fit: two buffers of nine populations and the coefficients, for two tiles.
 __host__ __device__ constexpr int tl_cells(int nc) { return nc == 1 ? 1504 : (nc == 3 ? 1360 : (nc == 4 ? 1296 : 1184)); }
@@ -79,7 +81,7 @@ struct Tile {
 template <typename T, int COEF, bool GF, bool WALLS>
 __global__ void __launch_bounds__(TL_THREADS, 1) tiles_kernel(StepArgs<T, float> a, T *src, T *dst, TileGeom g, int steps,
                                                              int first_check, int check_every, unsigned *result,
-                                                             uint4 *exch, unsigned base, int *err)
+                                                             uint4 *exch, unsigned base, int *err, int patience)
 {
     constexpr int NC = ncoef<COEF, GF>(), NP = tl_cells(NC), HALO = TILE_HALO;
     extern __shared__ __align__(16) unsigned char tl_raw[];
@@ -219,7 +221,7 @@ __global__ void __launch_bounds__(TL_THREADS, 1) tiles_kernel(StepArgs<T, float>
 #pragma unroll
                 for (int w = 0; w < 3; ++w) v[w] = tl_poll(area + w * cells + get_cell[j]);
                 if ((v[0].w == seq && v[1].w == seq && v[2].w == seq) || *(volatile int *)&s_failed) break;
-                if (++spins > TL_SPINS) {
+                if (++spins > patience) {
                     *(volatile int *)&s_failed = 1;
                     atomicExch(err, 1);
                 }
@@ -375,7 +377,8 @@ cudaError_t launch_tl(const StepArgs<T, float> &a, const TileGeom &g, const Tile
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, a, const_cast<T *>(a.src), a.dst, g, run.steps, run.first_check,
-                              run.check_every, run.result, static_cast<uint4 *>(run.exch), run.base, run.err);
+                              run.check_every, run.result, static_cast<uint4 *>(run.exch), run.base, run.err,
+                              run.patience);
 }
 
 template <typename T, int COEF>

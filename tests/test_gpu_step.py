@@ -466,3 +466,35 @@ def test_checks_inside_fused_passes_equal_single_steps_bitwise(storage, nx, ny, 
                 got.append(out)
         for a, b in zip(*got):
             np.testing.assert_array_equal(a, b)
+
+
+def test_resident_tiles_wait_that_runs_out_gives_etimeout():
+    """The blocks of a small lattice wait for one another's edges, at most for the time limit. With a limit of nothing the
+    first poll in vain gives up while every block goes on: the call returns LBM_ETIMEOUT, the grid refuses to step, to
+    read and to save until a state is loaded, and then goes on as if nothing had happened."""
+    import torch
+    lbm = _lbm()
+    kap = torch.from_numpy(synth.lognormal_kappa(257, 255, 4.0, 1.5, seed=31).astype(np.float32)).cuda()
+    p = lbm.Params(nx=257, ny=255, tau=0.7, gx=1e-6, gy=3e-7)
+    with lbm.Grid(p, kap) as G:
+        G.step(40)
+        st = torch.empty(lbm.lbm_grid_state_bytes(G.handle), dtype=torch.uint8, device="cuda")
+        t = lbm.lbm_grid_save_state(G.handle, st)
+        G.step(200, 0.0, 50)
+        ref = [f.cpu() for f in G.fields()]
+        try:
+            lbm.lbm_set_time_limit(1e-10)
+            with pytest.raises(lbm.LbmError) as ei:
+                G.step(200, 0.0, 50)
+            assert ei.value.status == lbm.LBM_ETIMEOUT
+        finally:
+            lbm.lbm_set_time_limit(600.0)
+        for call in (lambda: G.step(1), G.fields, lambda: lbm.lbm_mean_velocity(G.handle),
+                     lambda: lbm.lbm_grid_save_state(G.handle, st)):
+            with pytest.raises(lbm.LbmError) as ei:
+                call()
+            assert ei.value.status == lbm.LBM_ETIMEOUT
+        lbm.lbm_grid_load_state(G.handle, st, t)
+        G.step(200, 0.0, 50)
+        for a, b in zip(G.fields(), ref):
+            assert torch.equal(a.cpu(), b)
