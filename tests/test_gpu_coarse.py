@@ -210,3 +210,37 @@ def test_coarse_run_fused_passes_equal_single_steps_bitwise(nx, ny, monkeypatch)
                 got.append(out)
             for a, b in zip(*got):
                 assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("nx,ny", [(777, 401), (1024, 520), (35001, 9)])
+def test_coarse_run_of_large_lattices_equals_single_steps_bitwise(nx, ny, monkeypatch):
+    """Coarse lattices too large to stay in shared memory go through passes of up to four steps, the tensor drag with and
+    without a force field, walls, odd columns and few rows; fixed steps, with checks inside and beside a pass, and a
+    stop at the tolerance. Fields and the step count equal the one-step kernel's."""
+    import torch
+    import paper_1312_0195_gb300 as lbm
+    g = torch.Generator().manual_seed(nx)
+    K = 0.05 * torch.rand((ny, nx, 4), generator=g, dtype=torch.float64)
+    K[..., 0] += 0.2
+    K[..., 3] += 0.2
+    K = K.cuda()
+    field = torch.rand((2, ny, nx), generator=g).cuda() * 1e-6
+    for bc in (lbm.LBM_BC_PERIODIC, lbm.LBM_BC_WALLS_Y):
+        for force in (None, field):
+            got = []
+            for single in (False, True):
+                if single:
+                    monkeypatch.setenv("LBM_STEP_VEC", "1")
+                else:
+                    monkeypatch.delenv("LBM_STEP_VEC", raising=False)
+                runs = []
+                for steps, tol, check in ((77, 0.0, 0), (77, 0.0, 19), (130, 0.0, 64), (400, 0.03, 13)):
+                    out = [torch.empty((ny, nx), device="cuda") for _ in range(3)]
+                    _, n = lbm.lbm_coarse_run(lbm.Params(nx=4 * nx, ny=4 * ny, tau=1.0, gx=1e-6, bc=bc), 4, K, force, steps,
+                                              tol, check, *out)
+                    runs.append((n, out))
+                got.append(runs)
+            for (n, a), (m, b) in zip(*got):
+                assert n == m
+                for x, y in zip(a, b):
+                    assert torch.equal(x, y)

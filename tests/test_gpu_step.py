@@ -498,3 +498,32 @@ def test_resident_tiles_wait_that_runs_out_gives_etimeout():
         G.step(200, 0.0, 50)
         for a, b in zip(G.fields(), ref):
             assert torch.equal(a.cpu(), b)
+
+
+@pytest.mark.parametrize("storage", [0, 1])
+@pytest.mark.parametrize("nx,ny", [(777, 401), (35001, 9), (35000, 8), (57, 6001)])
+def test_long_fused_runs_of_large_lattices_equal_single_steps_bitwise(storage, nx, ny, monkeypatch):
+    """Long runs in passes of up to four steps, on lattices that do not fit into shared memory: odd columns with and
+    without walls and a force field, as few rows as a pass takes, and one strip and one column. States and residuals agree
+    with single steps bit for bit."""
+    import torch
+    lbm = _lbm()
+    kap = torch.from_numpy(synth.lognormal_kappa(nx, ny, 4.0, 1.5, seed=nx + ny).astype(np.float32)).cuda()
+    field = torch.rand((2, ny, nx), generator=torch.Generator().manual_seed(3)).cuda() * 1e-6
+    for walls in (False, True):
+        for force in (None, field):
+            got = []
+            for single in (False, True):
+                if single:
+                    monkeypatch.setenv("LBM_STEP_VEC", "1")
+                else:
+                    monkeypatch.delenv("LBM_STEP_VEC", raising=False)
+                p = lbm.Params(nx=nx, ny=ny, tau=0.7, gx=1e-6, gy=3e-7, storage=storage,
+                               bc=lbm.LBM_BC_WALLS_Y if walls else lbm.LBM_BC_PERIODIC)
+                with lbm.Grid(p, kap, force) as G:
+                    resid = [G.step(n, 0.0, check)[1] for n, check in ((130, 64), (103, 0), (61, 7))]
+                    st = torch.empty(lbm.lbm_grid_state_bytes(G.handle), dtype=torch.uint8, device="cuda")
+                    lbm.lbm_grid_save_state(G.handle, st)
+                    got.append((resid, st.cpu().numpy()))
+            assert got[0][0] == got[1][0]
+            np.testing.assert_array_equal(got[0][1], got[1][1])
