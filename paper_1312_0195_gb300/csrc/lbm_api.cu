@@ -523,7 +523,9 @@ lbm_status grid_create_impl(const lbm_params *p, const float *kappa_dev, const d
     // launch shapes: persistent step grid, fixed moment grid (fixed reduction order)
     const int sms = sm_count(g->dev);
     g->sms = sms;
-    g->fused = !std::getenv("LBM_STEP_VEC") && multistep_ok(p->storage, g->coef_mode, p->nx, p->ny, p->force_model);
+    const bool several = !std::getenv("LBM_STEP_VEC") &&
+                         multistep_ok(p->storage, g->coef_mode, p->nx, p->ny, p->force_model);
+    g->fused = several && multistep_pays(p->storage, p->nx, p->ny, sms);
     const int vec = step_vec(p->storage, p->nx);
     const int64_t chunks = n / vec;
     const bool f64 = p->storage == LBM_F64;
@@ -552,7 +554,7 @@ lbm_status grid_create_impl(const lbm_params *p, const float *kappa_dev, const d
     const int64_t mcap = (int64_t)sms * 2;   // 128 registers: two 256-thread blocks per SM
     g->L.mom_blocks = (int)(mwant < mcap ? (mwant < 1 ? 1 : mwant) : mcap);
 
-    if (g->fused) g->tiles = tile_geometry(p->storage, g->coef_mode, g->has_g, p->nx, p->ny, sms);
+    if (several) g->tiles = tile_geometry(p->storage, g->coef_mode, g->has_g, p->nx, p->ny, sms);
     // One allocation for everything, zeroed in one go: with one each, a memset each, a capture stream and pinned
     // memory a coarse run of 1250 steps on 256 x 256 took 2.3 ms instead of 1.8. No room for the exchanges of the
     // tile kernel: stepped in passes over memory.

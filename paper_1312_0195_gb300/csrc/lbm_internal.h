@@ -80,6 +80,7 @@ constexpr int MULTISTEP_MAX = 4;        // steps one pass fuses at most
 constexpr int MULTISTEP_MIN_ROWS = 4;   // rows of a warp's segment at least: fewer repeat more halo rows than
                                         // they gain in parallel warps (256 x 256: 2.9 us a step at 4, 3.3 at 2)
 bool multistep_ok(int storage, int coef_mode, int nx, int ny, int guo);
+bool multistep_pays(int storage, int nx, int ny, int sms);
 cudaError_t launch_multistep(int storage, int coef_mode, bool gfield, bool walls, const void *args, int nlev, int sms,
                              unsigned *check, cudaStream_t st);
 

@@ -27,6 +27,7 @@
 #include "lbm_internal.h"
 #include "pair_step.cuh"
 
+#include <algorithm>
 #include <type_traits>
 
 namespace lbm {
@@ -410,14 +411,48 @@ cudaError_t launch_c(bool gf, bool walls, const StepArgs<T, float> &a, int nlev,
 }  // namespace
 
 // Guo's scheme and FP16 with a tensor K* keep the one-step kernel; so do lattices too small for the
-// single wrap of a row index. Elsewhere a fused pass was faster at every size measured (us a step; 128 x 64:
-// 2.0 against 2.6; 517 x 389, odd rows: 2.9 against 4.0; 4096 x 4096: 53 against 196). Long runs of small
-// lattices go on to tiles.cu.
+// single wrap of a row index.
 bool multistep_ok(int storage, int coef_mode, int nx, int ny, int guo)
 {
     if ((int64_t)nx * ny >= (int64_t)1 << 30) return false;      // 32-bit byte offsets within a plane
     if (guo || ny < 2 * LEV || nx < 2) return false;
     return storage == LBM_F32 || (storage == LBM_F16 && coef_mode == COEF_SCALAR);
+}
+
+// Whether passes of four steps beat single steps, by microseconds a step of either. A pass takes the longest warp's
+// march: its positions (rows, and 2 (LEV - 1) of halo), each dearer the more warps share an SM, whatever part of a
+// strip's columns the lattice fills. A single step takes a launch and its bytes' way, from L2 up to about a million
+// cells. Against 526 measured pairs (both storages, 2 to 131,073 columns, 8 to 400,000 rows, 16 to 29 M cells) the
+// choice is at worst 1.13 times the better one, where passes everywhere were up to 17 times it: 2 x 1,048,576 cells 370 us
+// a step against 33, 24 x 65,536 in FP16 14.3 against 8.2, 64 x 16,384 in FP16 8.6 against 6.4, 400 x 1000 in FP16
+// 4.6 against 4.1. Passes win at 128 x 64 (2.0 against 2.6), 517 x 389 (2.9 against 4.0), 1448 x 1448 (8.9 against
+// 24.2) and 4096 x 4096 (53 against 196). Long runs of small lattices go on to tiles.cu.
+bool multistep_pays(int storage, int nx, int ny, int sms)
+{
+    if (nx < 4) return false;
+    const bool f16 = storage == LBM_F16, odd = nx % 2 != 0;
+    const int warps = f16 ? ms_warps<__half>() : ms_warps<float>();
+    const int strips = (nx + USEFUL - 1) / USEFUL;
+    const int64_t segs = std::max<int64_t>(1, (int64_t)sms * warps / strips);
+    const int64_t rows = std::max<int64_t>(MULTISTEP_MIN_ROWS, (ny + segs - 1) / segs);
+    double load = (double)strips * ((ny + rows - 1) / rows) / sms;          // warps on an SM
+    load = load > 12.0 ? 16.0 : std::max(load, 1.0);                        // four schedulers
+    const double positions = (double)((rows + 2 * (LEV - 1) + 1) / 2 * 2);
+    const double fixed = odd ? (f16 ? 0.90 : 0.34) : (f16 ? 0.36 : 0.38), shared = odd ? (f16 ? 0.075 : 0.077) : (f16 ? 0.078 : 0.061);
+    const double pass = (fixed + shared * load) * positions + (odd ? (f16 ? 0.0 : 3.5) : 2.5);
+
+    const double n = 1e-6 * nx * ny;                                        // million cells
+    double single;
+    if (nx % (f16 ? 8 : 4) == 0) {
+        if (n < 6e-4) single = 1.8;
+        else if (f16) single = n < 2.3 ? 2.9 + 3.4 * n : 7.2 * n;
+        else single = n < 1.4 ? 2.5 + 5.6 * n : 12.2 * n;
+    } else if (f16 && !odd) {
+        single = nx % 4 == 0 && n >= 1.05 && n < 2.3 ? 2.9 + 4.3 * n : 2.0 + 7.2 * n;
+    } else {
+        single = f16 || n < 1.4 ? (f16 ? 1.80 : 1.95) + 11.7 * n : 14.7 * n;
+    }
+    return pass < LEV * single;
 }
 
 cudaError_t launch_multistep(int storage, int coef_mode, bool gfield, bool walls, const void *args, int nlev, int sms,

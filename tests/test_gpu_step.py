@@ -501,7 +501,7 @@ def test_resident_tiles_wait_that_runs_out_gives_etimeout():
 
 
 @pytest.mark.parametrize("storage", [0, 1])
-@pytest.mark.parametrize("nx,ny", [(777, 401), (35001, 9), (35000, 8), (57, 6001)])
+@pytest.mark.parametrize("nx,ny", [(777, 401), (35001, 9), (35000, 8), (57, 6001), (1002, 700)])
 def test_long_fused_runs_of_large_lattices_equal_single_steps_bitwise(storage, nx, ny, monkeypatch):
     """Long runs in passes of up to four steps, on lattices that do not fit into shared memory: odd columns with and
     without walls and a force field, as few rows as a pass takes, and one strip and one column. States and residuals agree
@@ -527,3 +527,20 @@ def test_long_fused_runs_of_large_lattices_equal_single_steps_bitwise(storage, n
                     got.append((resid, st.cpu().numpy()))
             assert got[0][0] == got[1][0]
             np.testing.assert_array_equal(got[0][1], got[1][1])
+
+
+@pytest.mark.parametrize("storage,nx,ny,passes", [
+    (0, 4096, 512, True), (1, 4096, 512, True), (0, 777, 401, True), (1, 777, 401, True), (0, 35001, 9, True),
+    (0, 32, 40000, True), (0, 58, 20000, True), (0, 2, 200000, False), (0, 4, 100000, False), (0, 7, 70001, False),
+    (0, 12, 40000, False), (1, 8, 60000, False), (1, 24, 65536, False), (1, 64, 16384, False), (1, 400, 1000, False)])
+def test_passes_of_several_steps_where_they_pay(storage, nx, ny, passes):
+    """A strip of a pass is 64 columns wide whatever the lattice: tall narrow lattices, and FP16 lattices of which an L2
+    holds the state, are stepped one by one, as they are faster so. 64 steps are 64 launches then, 17 otherwise (the last
+    is a single step). None of these lattices fits into shared memory."""
+    import torch
+    lbm = _lbm()
+    kap = torch.full((ny, nx), 1e-2, device="cuda")
+    with lbm.Grid(lbm.Params(nx=nx, ny=ny, tau=0.8, gx=1e-6, storage=storage), kap) as G:
+        n = lbm.lbm_launch_count()
+        G.step(64)
+        assert lbm.lbm_launch_count() - n == (17 if passes else 64)
