@@ -686,7 +686,7 @@ lbm_status lbm_step(lbm_grid *g, int64_t max_steps, double tol_rel, int32_t chec
         // one launch of the tile kernel runs up to the next value the host needs
         int64_t m = left < TILE_CHUNK ? left : TILE_CHUNK;
         if (tol_rel > 0.0) m = std::min<int64_t>(m, check_every - g->t % check_every);
-        if (g->tiles.ntx > 0 && m >= TILES_FROM) {
+        if (g->tiles.ntx > 0 && m >= tiles_from(g->tiles)) {
             int checks = 0;
             const cudaError_t e = enqueue_tiles(g, (int)m, check_every, &checks);
             if (e == cudaErrorCooperativeLaunchTooLarge) {       // a stream with a part of the SMs

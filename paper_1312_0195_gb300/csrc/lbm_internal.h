@@ -93,9 +93,12 @@ struct TileGeom {
 };
 TileGeom tile_geometry(int storage, int coef_mode, bool gfield, int nx, int ny, int sms);
 // Steps of a launch at least (more than TILE_HALO: an exchange has to take place). Filling shared memory, writing it
-// back and reading the outcome cost about 20 us. Microseconds of a call here / in passes of four: 12 steps 31 / 33 at
-// 128 x 64, 46 / 47 at 517 x 389, 52 / 44 at 500 x 500, the largest; 16 steps 60 / 55 and 24 steps 77 / 76 there.
-constexpr int TILES_FROM = 16;
+// back and reading the outcome cost about 20 us, and a step of the largest arrays almost as much as in passes of four.
+// Microseconds of a call here / in passes: 12 steps 30 / 32 and 16 steps 32 / 39 at 128 x 64 (arrays of 256 cells), 16
+// steps 41 / 39 and 20 steps 43 / 47 at 256 x 256 (528), 12 steps 52 / 47 and 16 steps 55 / 59 at 517 x 389 (1156), 16
+// steps 53 / 53 and 24 steps 67 / 74 at 480 x 480 (1280); 16 steps 66 / 54, 28 steps 90 / 86 and 32 steps 93 / 96 at
+// 500 x 500 (1386), 28 steps 90 / 86 and 40 steps 118 / 118 at 500 x 540 (1452).
+inline int tiles_from(const TileGeom &g) { return g.W * g.H > 1300 ? 32 : 16; }
 constexpr double TILE_POLLS = 2.1e6;    // polls of a thread in a second at most: a round trip to L2 each
 constexpr size_t tile_exchange_bytes(int64_t cells) { return (size_t)cells * 2 * 3 * 16; }
 // One launch: `steps` steps from the state in src, with the residual's maxima (bits of max |du| and max |u|) after

@@ -544,3 +544,17 @@ def test_passes_of_several_steps_where_they_pay(storage, nx, ny, passes):
         n = lbm.lbm_launch_count()
         G.step(64)
         assert lbm.lbm_launch_count() - n == (17 if passes else 64)
+
+
+@pytest.mark.parametrize("nx,ny,steps,resident", [(128, 64, 15, False), (128, 64, 16, True), (480, 480, 16, True),
+                                                  (500, 500, 31, False), (500, 500, 32, True)])
+def test_runs_that_go_to_shared_memory(nx, ny, steps, resident):
+    """The shortest run of a small lattice that is stepped in shared memory, in one launch: 16 steps, and 32 on the largest
+    lattices, whose shorter runs are faster in passes."""
+    import torch
+    lbm = _lbm()
+    kap = torch.full((ny, nx), 1e-2, device="cuda")
+    with lbm.Grid(lbm.Params(nx=nx, ny=ny, tau=0.8, gx=1e-6), kap) as G:
+        n = lbm.lbm_launch_count()
+        G.step(steps)
+        assert (lbm.lbm_launch_count() - n == 1) == resident
