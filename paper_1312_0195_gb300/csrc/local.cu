@@ -94,7 +94,8 @@ struct LocalArgs {
     int *worst;               // [1] (zeroed)
     int *abort_flag;          // [1] (zeroed)
     unsigned long long time_limit_ns;
-    unsigned long long *t_start;   // [1] when the call's first CTA started (zeroed), or nullptr: each launch its own
+    unsigned long long *t_start;   // [1] complement of the call's earliest start (zeroed), or nullptr: each CTA its own
+    int wave;                 // CTAs of the shared-memory solver that start together
     int skip_reg;             // 1: sides of the register solver (local_reg.cuh) are not taken here
 };
 
@@ -112,11 +113,18 @@ __device__ __forceinline__ unsigned long long globaltimer()
     return t;
 }
 
-// the start of the wall-clock limit, the same for every CTA of a call's launches
-__device__ __forceinline__ unsigned long long start_time(const LocalArgs &a)
+// The wall-clock limit counts from the first start of a CTA of the call's launches: each notes its own, and a check
+// reads the earliest.
+__device__ __forceinline__ unsigned long long note_start(const LocalArgs &a)
 {
-    const unsigned long long now = globaltimer(), first = a.t_start ? atomicCAS(a.t_start, 0ull, now) : 0ull;
-    return first ? first : now;
+    const unsigned long long now = globaltimer();
+    if (a.t_start) atomicMax(a.t_start, ~now);
+    return now;
+}
+__device__ __forceinline__ bool past_limit(const LocalArgs &a, unsigned long long own)
+{
+    const unsigned long long first = a.t_start ? ~*(volatile unsigned long long *)a.t_start : own;
+    return globaltimer() - first > a.time_limit_ns;
 }
 
 // drag fraction e = 1 - d = eps nu / (2 kappa + eps nu) of Eq. 6 (see the fine-grid step)
@@ -672,28 +680,37 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) local_keff_kernel(LocalArgs 
 
     __shared__ int s_nclass, s_csize[MAXCLASS], s_coff[MAXCLASS], s_cend[MAXCLASS], s_chead[MAXCLASS];
     __shared__ unsigned long long s_t0;
+    __shared__ float s_fill;                  // part of all CTAs' slots that the batch takes
 
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const T hg = kc<T>(a, K_HG);
     if (tid == 0) {
-        s_t0 = start_time(a);
+        s_t0 = note_start(a);
         s_abort = 0;
         // this solver's classes (a table is built on the device by an earlier kernel of the same stream). Skipping the
         // others here and not in the loop keeps a branch out of it that slowed every step by 3 %.
         const int nc = a.table ? (a.table[DT_BAD] ? 0 : a.table[DT_NCLASS]) : a.nclass;
         int k = 0;
+        float hold = 0.0f;
         for (int c = 0; c < nc; ++c) {
             const int s = a.table ? a.table[DT_SIZE + c] : a.class_size[c];
             if (a.skip_reg && reg_side(s)) continue;
             s_csize[k] = s;
             s_coff[k] = a.table ? a.table[DT_OFF + c] : a.class_off[c];
             s_cend[k] = a.table ? a.table[DT_OFF + c + 1] : a.class_off[c + 1];
+            hold += (float)(s_cend[k] - s_coff[k]) / min(CMAX / (s * s), MAXSLOTS);
             s_chead[k++] = c;
         }
         s_nclass = k;
+        s_fill = fminf(1.0f, hold / a.wave);
     }
     __syncthreads();
 
+    // A batch that the CTAs together hold with room to spare is spread over all of them, each taking the same part of what
+    // it holds; else the first CTAs to come take as many jobs as they hold and the others none. 1000 steps, ms: 40 FP64
+    // leaves of 8 cells 2.1 instead of 18.8, 200 leaves of 15 cells 1.05 instead of 2.5. A CTA that has worked on another
+    // size takes all it can.
+    bool worked = false;
     for (int cls = 0; cls < s_nclass; ++cls) {
         const int s = s_csize[cls], s2 = s * s;
         int nslots = CMAX / s2;
@@ -720,7 +737,8 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) local_keff_kernel(LocalArgs 
             Slot sl;
             sl.job = -1;
             const int qbeg = s_coff[cls], qn = s_cend[cls] - qbeg;
-            int q = s_abort ? qn : atomicAdd(&a.heads[s_chead[cls]], 1);
+            const int take = worked ? nslots : max(1, (int)ceilf(nslots * s_fill));
+            int q = s_abort || tid >= take ? qn : atomicAdd(&a.heads[s_chead[cls]], 1);
             if (q < qn) {
                 sl.job = a.jobs[qbeg + q];
                 sl.leaf = sl.job >> 1;
@@ -793,7 +811,7 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) local_keff_kernel(LocalArgs 
             if ((int)(Tcta - s_event) <= 0 && (Tcta & 255u) != 0) continue;
             if (tid == 0 && !s_abort) {
                 if (*(volatile int *)a.abort_flag) s_abort = 1;
-                else if (globaltimer() - s_t0 > a.time_limit_ns) {
+                else if (past_limit(a, s_t0)) {
                     s_abort = 1;
                     atomicExch(a.abort_flag, 1);
                 }
@@ -948,6 +966,7 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) local_keff_kernel(LocalArgs 
             }
             fresh = __syncthreads_or(tid < nslots && (hot[tid].z & 4)) != 0;
         }
+        worked |= Tcta > 0;
     }
     // started beside the register solver (launch_solvers): whoever waits for this kernel waits for that one too
     if (tid == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1109,9 +1128,9 @@ __global__ void __launch_bounds__(256) abandon_kernel(LocalArgs a, int reg_block
 // and their time for a step (1.3 and 2.2 us), so that short lists of either do not wait; CTAs of the second take
 // over SMs that the first gives back.
 // Milliseconds in the shared-memory solver alone / one launch after the other / side by side:
-// one leaf of every side from 1 to 40, 2000 steps 3.6 / 6.0 / 3.7, to the tolerance 34 / 52 / 35; fifty of each, 1000
-// steps 9.7 / 10.5 / 9.9; twenty of each, to the tolerance 82 / 131 / 84; 4000 leaves of 16 cells and 40 of 15, to the
-// tolerance 47 / 37 / 22, 40 and 4000 43 / 51 / 44. With SMs by cells alone, twenty of each took 99.
+// one leaf of every side from 1 to 40, 2000 steps 3.6 / 6.0 / 2.6, to the tolerance 34 / 52 / 35; fifty of each, 1000
+// steps 9.7 / 10.5 / 9.7; twenty of each, to the tolerance 82 / 131 / 83; 4000 leaves of 16 cells and 40 of 15, to the
+// tolerance 47 / 37 / 23, 40 and 4000 43 / 51 / 42. With SMs by cells alone, twenty of each took 99.
 cudaError_t launch_solvers(LocalArgs &a, bool f64, double tau, bool lg, int sms, bool reg, bool other,
                            cudaStream_t st)
 {
@@ -1141,6 +1160,7 @@ cudaError_t launch_solvers(LocalArgs &a, bool f64, double tau, bool lg, int sms,
     }
     if (!use_reg || other) {
         a.skip_reg = use_reg ? 1 : 0;
+        a.wave = std::max(1, std::min(blocks, sms - reg_blocks));
         const LocalKernel kern = lg ? local_kernel_lg(f64, tau) : local_kernel(f64, tau, a.warm);
         const size_t smem = lg ? (f64 ? lg_smem<double>() : lg_smem<float>())
                                : f64 ? LocalCfg<double>::SMEM : LocalCfg<float>::SMEM;
