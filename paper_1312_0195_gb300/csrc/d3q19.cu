@@ -26,6 +26,7 @@ namespace lbm {
 lbm_status fail(lbm_status s, const char *fmt, ...);
 bool is_device_ptr(const void *p);
 void count_launches(int64_t n);
+int sm_count(int dev);
 
 namespace {
 
@@ -1082,52 +1083,140 @@ lbm_status cluster_result(const unsigned long long *d_clock, cudaStream_t st)
     return LBM_OK;
 }
 
-// The same two jobs at a time (local3_pair.cuh): FP32 cubes of at most CP3_MAX_SIDE cells a side, whose slabs take
-// clusters of at most 6 CTAs. LBM_EINVAL (nothing launched) for other cubes, or if the device cannot schedule
-// such a cluster. Measured on batches that fill the chip, billions of updates a second, one job a cluster -> two:
-// side 8 136 -> 160, 10 118 -> 122, 12 98 -> 122, 14 91 -> 97, 16 109 -> 120, 18 78 -> 97.
-lbm_status run_pair_size(const lbm3d_params *p, const float *kappa_dev, const int4 *d_l4, const std::vector<int> &ids,
-                         int *d_ids, int sz, int m, double nu, double g_const, double tol_rel, int64_t max_steps,
-                         int32_t check_every, int optin, unsigned long long *d_clock, double *keff_dev,
-                         int32_t *status_dev, int32_t *steps_dev, cudaStream_t st)
+// How cubes of one side go onto clusters: CTAs of a cluster, layers of a CTA's slab, threads, and the clusters that the
+// chip holds at once.
+struct CluPlan {
+    int C = 0, L = 0, nt = 0, clusters = 0;
+    size_t smem = 0;
+    const void *fn = nullptr;
+};
+cudaLaunchConfig_t cluster_config(const CluPlan &pl, cudaLaunchAttribute *attr, cudaStream_t st)
 {
-    if (p->storage != LBM_F32 || sz > CP3_MAX_SIDE || ids.size() > (size_t)INT_MAX / 3 - 1) return LBM_EINVAL;
-    const int s2 = sz * sz;
-    int C = 0, L = 0;
-    // slabs of at most 512 cells (two CTAs on an SM cover each other's barriers) where they take at most 4 CTAs,
-    // else of at most 1024 (side 12: 122 against 111 billion updates a second; 16, with 8 CTAs: 103 against 120)
-    for (int cells : {512, CP3_THREADS * CP3_CPT}) {
-        const int lmax = std::max(1, cells / s2), c = (sz + lmax - 1) / lmax;
-        L = (sz + c - 1) / c;
-        C = (sz + L - 1) / L;
-        if (C <= 4) break;
-    }
-    const int P = L * s2;
-    const int PS = P <= 256 ? 256 : (P <= 512 ? 512 : 1024);
-    const size_t smem = pair3_smem_bytes(PS);
-    const void *fn = pair3_kernel(PS);
-    if (smem > (size_t)optin) return LBM_EINVAL;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-        cudaGetLastError();
-        return LBM_EINVAL;
-    }
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)C;
+    attr[0].val.clusterDim.x = (unsigned)pl.C;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
-    cfg.blockDim = dim3((unsigned)std::min(CP3_THREADS, ((P + CP3_CPT - 1) / CP3_CPT + 31) / 32 * 32));
-    cfg.dynamicSmemBytes = smem;
+    cfg.gridDim = dim3((unsigned)pl.C);
+    cfg.blockDim = dim3((unsigned)pl.nt);
+    cfg.dynamicSmemBytes = pl.smem;
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cfg.gridDim = dim3((unsigned)C);
-    int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) != cudaSuccess || nclusters < 1) {
-        cudaGetLastError();
-        return LBM_EINVAL;
+    return cfg;
+}
+bool cluster_room(CluPlan &pl)
+{
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = cluster_config(pl, attr, nullptr);
+    if (cudaOccupancyMaxActiveClusters(&pl.clusters, pl.fn, &cfg) == cudaSuccess && pl.clusters >= 1) return true;
+    cudaGetLastError();
+    return false;
+}
+
+// One job a cluster: the fewest CTAs whose slab of L s^2 cells fits a compiled slot stride PS.
+bool one_job_plan(bool f64, int sz, int optin, CluPlan &pl)
+{
+    const size_t esz = f64 ? 8 : 4;
+    const int NT = f64 ? clu3_threads<double>() : clu3_threads<float>();
+    const int CPT = f64 ? clu3_cpt<double>() : clu3_cpt<float>();
+    if (sz > 32) return false;
+    int PS = 0;
+    for (int c = 1; c <= 16 && c <= sz && PS == 0; c *= 2) {
+        const int l = (sz + c - 1) / c;
+        const int64_t P = (int64_t)l * sz * sz;
+        for (int ps : {256, 512, 1024, 2048}) {
+            if (P <= ps && P <= (int64_t)CPT * NT && clu3_smem_bytes(ps, esz) <= (size_t)optin &&
+                (!f64 || ps <= 1024)) {
+                pl.C = c;
+                pl.L = l;
+                PS = ps;
+                break;
+            }
+        }
     }
+    if (PS == 0) return false;
+    const int64_t P = (int64_t)pl.L * sz * sz;
+    pl.smem = clu3_smem_bytes(PS, esz);
+    // enough threads for CPT cells each, whole warps
+    pl.nt = (int)std::min<int64_t>(NT, ((P + CPT - 1) / CPT + 31) / 32 * 32);
+    pl.fn = f64 ? clu3_kernel<double>(PS) : clu3_kernel<float>(PS);
+    if (!pl.fn) return false;
+    // the opt-in maximum, not this launch's size: a concurrent call with a larger cube stays valid
+    if (cudaFuncSetAttribute(pl.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess ||
+        (pl.C > 8 && cudaFuncSetAttribute(pl.fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
+        cudaGetLastError();
+        return false;
+    }
+    return cluster_room(pl);
+}
+
+// Two jobs a cluster: slabs of at most 512 cells (two CTAs on an SM cover each other's barriers) where they take at most
+// 4 CTAs, else of at most 1024 (side 12: 122 against 111 billion updates a second; 16, with 8 CTAs: 103 against 120).
+bool pair_plan(int sz, int optin, CluPlan &pl)
+{
+    if (sz > CP3_MAX_SIDE) return false;
+    const int s2 = sz * sz;
+    for (int cells : {512, CP3_THREADS * CP3_CPT}) {
+        const int lmax = std::max(1, cells / s2), c = (sz + lmax - 1) / lmax;
+        pl.L = (sz + c - 1) / c;
+        pl.C = (sz + pl.L - 1) / pl.L;
+        if (pl.C <= 4) break;
+    }
+    const int P = pl.L * s2;
+    const int PS = P <= 256 ? 256 : (P <= 512 ? 512 : 1024);
+    pl.smem = pair3_smem_bytes(PS);
+    pl.fn = pair3_kernel(PS);
+    pl.nt = std::min(CP3_THREADS, ((P + CP3_CPT - 1) / CP3_CPT + 31) / 32 * 32);
+    if (pl.smem > (size_t)optin) return false;
+    if (cudaFuncSetAttribute(pl.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return cluster_room(pl);
+}
+
+// Whether two jobs a cluster beat one. Time of a batch in units of a lone cluster's step with one job: whole rounds of
+// the jobs that the chip holds, and the rest, each by the CTAs that share an SM (a CTA of 512 cells slows its
+// neighbours' steps by 0.33, with two jobs by 0.5). A lone cluster's step with two jobs: 1.08, where it has at least
+// twice the CTAs 0.88 for twice, 0.76 for three and 0.64 for four times as many (12 cells), and 0.85 at 5 and 6 cells,
+// whose slabs get twice the threads; a check costs 7.5 such steps against 4.5. Over sides 1 to 18 and 14 batches of
+// 1 to 450 cubes, 500 steps, the choice is at worst 1.03 times one job a cluster, where two jobs everywhere were up to
+// 1.65 times it (25 cubes of 15 cells 2.7 ms against 1.6, 50 of 16 3.8 against 3.1, 50 of 8 1.00 against 0.90). Batches
+// that fill the chip, billions of updates a second, one job -> two: side 8 136 -> 160, 10 118 -> 122, 12 98 -> 122,
+// 14 91 -> 97, 16 109 -> 120, 18 78 -> 97.
+bool pair_pays(const CluPlan &one, const CluPlan &two, int sz, int64_t njobs, int32_t check_every, int sms)
+{
+    auto rounds = [&](const CluPlan &pl, int per, double slope) {
+        auto share = [&](int64_t jobs) {
+            const int64_t ctas = (jobs + per - 1) / per * pl.C, on_sm = std::max<int64_t>(1, (ctas + sms - 1) / sms);
+            return 1.0 + slope * pl.L * sz * sz / 512.0 * (double)(on_sm - 1);
+        };
+        const int64_t hold = (int64_t)pl.clusters * per, full = njobs / hold, rest = njobs - full * hold;
+        return (double)full * share(hold) + (rest ? share(rest) : 0.0);
+    };
+    const int cells = sz * sz * sz, wider = two.C / one.C;
+    double step = wider >= 2 ? 1.12 - 0.12 * two.C / one.C : (cells > 64 && cells <= 256 ? 0.85 : 1.08);
+    step *= (1.0 + 7.5 / check_every) / (1.0 + 4.5 / check_every) / 1.044;
+    return step * rounds(two, 2, 0.5) < rounds(one, 1, 0.33);
+}
+
+// Runs every job of one leaf size two at a time (local3_pair.cuh): FP32 cubes of at most CP3_MAX_SIDE cells a side, where
+// that is the faster way. LBM_EINVAL (nothing launched) elsewhere, or if the device cannot schedule such a cluster.
+lbm_status run_pair_size(const lbm3d_params *p, const float *kappa_dev, const int4 *d_l4, const std::vector<int> &ids,
+                         int *d_ids, int sz, int m, double nu, double g_const, double tol_rel, int64_t max_steps,
+                         int32_t check_every, int optin, int sms, unsigned long long *d_clock, double *keff_dev,
+                         int32_t *status_dev, int32_t *steps_dev, cudaStream_t st)
+{
+    if (p->storage != LBM_F32 || ids.size() > (size_t)INT_MAX / 3 - 1) return LBM_EINVAL;
+    CluPlan pl, one;
+    if (!pair_plan(sz, optin, pl)) return LBM_EINVAL;
+    if (one_job_plan(false, sz, optin, one) && !pair_pays(one, pl, sz, 3 * (int64_t)ids.size(), check_every, sms))
+        return LBM_EINVAL;
+    const int C = pl.C, L = pl.L, nclusters = pl.clusters;
+    const void *fn = pl.fn;
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = cluster_config(pl, attr, st);
     const int n = (int)ids.size(), njobs = 3 * n;
     int *head = reinterpret_cast<int *>(d_clock + 2);
     if (cudaMemcpyAsync(d_ids, ids.data(), sizeof(int) * n, cudaMemcpyHostToDevice, st) != cudaSuccess ||
@@ -1161,55 +1250,12 @@ lbm_status run_cluster_size(const lbm3d_params *p, const float *kappa_dev, const
                             cudaStream_t st)
 {
     const bool f64 = p->storage == LBM_F64;
-    const size_t esz = f64 ? 8 : 4;
-    const int NT = f64 ? clu3_threads<double>() : clu3_threads<float>();
-    const int CPT = f64 ? clu3_cpt<double>() : clu3_cpt<float>();
-    if (sz > 32) return LBM_EINVAL;
-    // the fewest CTAs whose slab of L s^2 cells fits a compiled slot stride PS
-    int C = 0, L = 0, PS = 0;
-    for (int c = 1; c <= 16 && c <= sz && C == 0; c *= 2) {
-        const int l = (sz + c - 1) / c;
-        const int64_t P = (int64_t)l * sz * sz;
-        for (int ps : {256, 512, 1024, 2048}) {
-            if (P <= ps && P <= (int64_t)CPT * NT && clu3_smem_bytes(ps, esz) <= (size_t)optin &&
-                (!f64 || ps <= 1024)) {
-                C = c;
-                L = l;
-                PS = ps;
-                break;
-            }
-        }
-    }
-    if (C == 0) return LBM_EINVAL;
-    const int64_t P = (int64_t)L * sz * sz;
-    const size_t smem = clu3_smem_bytes(PS, esz);
-    // enough threads for CPT cells each, whole warps
-    const int nt = (int)std::min<int64_t>(NT, ((P + CPT - 1) / CPT + 31) / 32 * 32);
-    const void *fn = f64 ? clu3_kernel<double>(PS) : clu3_kernel<float>(PS);
-    if (!fn) return LBM_EINVAL;
-    // the opt-in maximum, not this launch's size: a concurrent call with a larger cube stays valid
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess ||
-        (C > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
-        cudaGetLastError();
-        return LBM_EINVAL;
-    }
-    cudaLaunchConfig_t cfg = {};
+    CluPlan pl;
+    if (!one_job_plan(f64, sz, optin, pl)) return LBM_EINVAL;
+    const int C = pl.C, L = pl.L;
+    const void *fn = pl.fn;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)C;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.blockDim = dim3((unsigned)nt);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cfg.gridDim = dim3((unsigned)C);
-    int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) != cudaSuccess || nclusters < 1) {
-        cudaGetLastError();
-        return LBM_EINVAL;
-    }
+    cudaLaunchConfig_t cfg = cluster_config(pl, attr, st);
     const int n = (int)ids.size();
     if (cudaMemcpyAsync(d_ids, ids.data(), sizeof(int) * n, cudaMemcpyHostToDevice, st) != cudaSuccess) {
         cudaGetLastError();
@@ -1612,7 +1658,7 @@ lbm_status lbm3d_local_keff_batch(const lbm3d_params *p, const float *kappa_dev,
         const int64_t s3 = (int64_t)sz * sz * sz;
         if (cluster_ok) {
             lbm_status cs = run_pair_size(p, kappa_dev, d_l4, kv.second, d_ids, sz, m, nu, g_const, tol_rel, max_steps,
-                                          check_every, optin, d_clock, keff_dev, status_dev, steps_dev, st);
+                                          check_every, optin, sm_count(dev), d_clock, keff_dev, status_dev, steps_dev, st);
             if (cs == LBM_EINVAL)
                 cs = run_cluster_size(p, kappa_dev, d_l4, kv.second, d_ids, sz, m, nu, g_const, tol_rel, max_steps,
                                       check_every, optin, d_clock, keff_dev, status_dev, steps_dev, st);

@@ -365,3 +365,19 @@ def test_local_keff3_time_limit_reaches_jobs_still_in_the_queue():
         assert worst == lbm.LBM_ETIMEOUT and n_notconv == 512
     finally:
         lbm.lbm_set_time_limit(600.0)
+
+
+@pytest.mark.parametrize("side,n", [(3, 450), (4, 450), (7, 300), (8, 300), (12, 130), (13, 84), (14, 84), (16, 134), (17, 50), (18, 50)])
+def test_local_keff3_batches_that_go_two_jobs_a_cluster_match_oracle(side, n):
+    """Small batches of most sides run one job to a cluster; these are large enough for two, with refills, and checked
+    like the batches above on a sample of their cubes."""
+    kap = _field(40, 40, 40, seed=81)
+    r = np.random.default_rng(side)
+    leaves = [(*r.integers(0, 41 - side, 3), side) for _ in range(n)]
+    ke, st, steps, _ = gpu_keff3(kap, leaves, 0.8, 0.1, 0.9, 1e-6, 0.0, 77, k=64)
+    assert (steps == 77).all() and (st == 0).all()
+    for i in [0, 1, n // 3, n // 2, n - 2, n - 1]:
+        x0, y0, z0, s = leaves[i]
+        cube = kap[z0:z0 + s, y0:y0 + s, x0:x0 + s].astype(np.float64)
+        ref = oracle.local_keff3(cube, 0.8, 0.1, 0.9, 1e-6, tol=0.0, max_steps=77, check_every=64)["keff"]
+        np.testing.assert_allclose(ke[i], ref, rtol=0, atol=1e-5 * np.abs(np.diag(ref)).max())
