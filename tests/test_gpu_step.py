@@ -558,3 +558,37 @@ def test_runs_that_go_to_shared_memory(nx, ny, steps, resident):
         n = lbm.lbm_launch_count()
         G.step(steps)
         assert (lbm.lbm_launch_count() - n == 1) == resident
+
+
+def test_small_lattices_of_several_threads_at_once():
+    """Four threads step small lattices of their own on streams of their own. One of them at a time has its blocks wait
+    for one another in shared memory, the others go through passes; every state is that of the same run alone."""
+    import threading
+
+    import torch
+    lbm = _lbm()
+    kaps = [torch.from_numpy(synth.lognormal_kappa(400, 300, 4.0, 1.0, seed=40 + i).astype(np.float32)).cuda() for i in range(4)]
+    p = lbm.Params(nx=400, ny=300, tau=0.8, gx=1e-6)
+
+    def run(i, stream):
+        with lbm.Grid(p, kaps[i], stream=stream) as G:
+            resid = [G.step(200, 0.0, 50)[1] for _ in range(10)]
+            st = torch.empty(lbm.lbm_grid_state_bytes(G.handle), dtype=torch.uint8, device="cuda")
+            lbm.lbm_grid_save_state(G.handle, st)
+            return resid, st.cpu().numpy()
+
+    ref = [run(i, None) for i in range(4)]
+    got = [None] * 4
+    streams = [torch.cuda.Stream() for _ in range(4)]
+
+    def work(i):
+        got[i] = run(i, streams[i].cuda_stream)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for a, b in zip(got, ref):
+        assert a[0] == b[0]
+        np.testing.assert_array_equal(a[1], b[1])
