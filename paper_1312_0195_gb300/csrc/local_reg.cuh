@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(RG_THREADS, 1) local_reg_kernel(LocalArgs a)
     RegShared &sh = *reinterpret_cast<RegShared *>(rg_smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
-        sh.t0 = note_start(a);
+        sh.t0 = start_time(a);
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the shared-memory solver needs nothing of this one
     }
     if (lane == 0) sh.abort[warp] = 0;
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(RG_THREADS, 1) local_reg_kernel(LocalArgs a)
             if (leader) {
                 if (lane == 0 && !sh.abort[q.w0]) {
                     if (*(volatile int *)a.abort_flag) sh.abort[q.w0] = 1;
-                    else if (past_limit(a, sh.t0)) {
+                    else if (globaltimer() - sh.t0 > a.time_limit_ns) {
                         sh.abort[q.w0] = 1;
                         atomicExch(a.abort_flag, 1);
                     }
