@@ -1178,27 +1178,30 @@ bool pair_plan(int sz, int optin, CluPlan &pl)
 
 // Whether two jobs a cluster beat one. Time of a batch in units of a lone cluster's step with one job: whole rounds of
 // the jobs that the chip holds, and the rest, each by the CTAs that share an SM (a CTA of 512 cells slows its
-// neighbours' steps by 0.33, with two jobs by 0.5). A lone cluster's step with two jobs: 1.08, where it has at least
-// twice the CTAs 0.88 for twice, 0.76 for three and 0.64 for four times as many (12 cells), and 0.85 at 5 and 6 cells,
-// whose slabs get twice the threads; a check costs 7.5 such steps against 4.5. Over sides 1 to 18 and 14 batches of
-// 1 to 450 cubes, 500 steps, the choice is at worst 1.03 times one job a cluster, where two jobs everywhere were up to
-// 1.65 times it (25 cubes of 15 cells 2.7 ms against 1.6, 50 of 16 3.8 against 3.1, 50 of 8 1.00 against 0.90). Batches
-// that fill the chip, billions of updates a second, one job -> two: side 8 136 -> 160, 10 118 -> 122, 12 98 -> 122,
-// 14 91 -> 97, 16 109 -> 120, 18 78 -> 97.
-bool pair_pays(const CluPlan &one, const CluPlan &two, int sz, int64_t njobs, int32_t check_every, int sms)
+// neighbours' steps by 0.33, with two jobs by 0.5); runs to a tolerance end one by one, and a tail of slow jobs, about
+// six rounds long, follows them alone. A lone cluster's step with two jobs costs 1.09, less where its CTAs have fewer
+// cells than with one (0.92 for half as many, 0.58 for a quarter: 12 cells), 0.85 at 5 and 6 cells, whose slabs get twice
+// the threads; a check costs 7.5 such steps against 4.5. Over sides 1 to 18, batches of 1 to 450 cubes of 500 steps and 37
+// batches to a tolerance, the choice is at worst 1.03 times one job a cluster, where two jobs everywhere were up to
+// 1.65 times it (25 cubes of 15 cells 2.7 ms against 1.6, 50 of 16 3.8 against 3.1, 64 of 8 to a tolerance 11.0 against
+// 9.6). Batches that fill the chip, billions of updates a second, one job -> two: side 8 136 -> 160, 10 118 -> 122,
+// 12 98 -> 122, 14 91 -> 97, 16 109 -> 120, 18 78 -> 97.
+bool pair_pays(const CluPlan &one, const CluPlan &two, int sz, int64_t njobs, double tol_rel, int32_t check_every, int sms)
 {
-    auto rounds = [&](const CluPlan &pl, int per, double slope) {
+    auto time = [&](const CluPlan &pl, int per, double slope) {
         auto share = [&](int64_t jobs) {
             const int64_t ctas = (jobs + per - 1) / per * pl.C, on_sm = std::max<int64_t>(1, (ctas + sms - 1) / sms);
             return 1.0 + slope * pl.L * sz * sz / 512.0 * (double)(on_sm - 1);
         };
         const int64_t hold = (int64_t)pl.clusters * per, full = njobs / hold, rest = njobs - full * hold;
+        if (tol_rel > 0.0) return (double)njobs / (double)hold * share(std::min(njobs, hold)) + 6.0;
         return (double)full * share(hold) + (rest ? share(rest) : 0.0);
     };
-    const int cells = sz * sz * sz, wider = two.C / one.C;
-    double step = wider >= 2 ? 1.12 - 0.12 * two.C / one.C : (cells > 64 && cells <= 256 ? 0.85 : 1.08);
+    const int cells = sz * sz * sz;
+    const double fewer = (double)one.L / two.L;
+    double step = fewer >= 1.5 ? 1.26 - 0.17 * fewer : (cells > 64 && cells <= 256 ? 0.85 : 1.09);
     step *= (1.0 + 7.5 / check_every) / (1.0 + 4.5 / check_every) / 1.044;
-    return step * rounds(two, 2, 0.5) < rounds(one, 1, 0.33);
+    return step * time(two, 2, 0.5) < time(one, 1, 0.33);
 }
 
 // Runs every job of one leaf size two at a time (local3_pair.cuh): FP32 cubes of at most CP3_MAX_SIDE cells a side, where
@@ -1211,7 +1214,7 @@ lbm_status run_pair_size(const lbm3d_params *p, const float *kappa_dev, const in
     if (p->storage != LBM_F32 || ids.size() > (size_t)INT_MAX / 3 - 1) return LBM_EINVAL;
     CluPlan pl, one;
     if (!pair_plan(sz, optin, pl)) return LBM_EINVAL;
-    if (one_job_plan(false, sz, optin, one) && !pair_pays(one, pl, sz, 3 * (int64_t)ids.size(), check_every, sms))
+    if (one_job_plan(false, sz, optin, one) && !pair_pays(one, pl, sz, 3 * (int64_t)ids.size(), tol_rel, check_every, sms))
         return LBM_EINVAL;
     const int C = pl.C, L = pl.L, nclusters = pl.clusters;
     const void *fn = pl.fn;
