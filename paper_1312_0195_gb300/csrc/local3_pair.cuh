@@ -10,8 +10,10 @@
 // come first), and the clusters stay for the whole batch. The arithmetic of a cell is the one-job kernel's,
 // operation by operation.
 //
-// What bounds it: the barrier that ends each step. Its release fence and the wait are 40 % of the stalls, and
-// loads, arithmetic and stores of a CTA's warps do not overlap (FMA pipe 32 %, shared memory 43 % busy at side 16).
+// What bounds it, at side 16: nothing is full. The shared-memory path is 56 % busy, the FMA pipe 41 %, issue slots 39 %;
+// the barrier that ends each step and its release fence are 17 % of the stalls, and loads, arithmetic and stores of a
+// CTA's warps, which start each step together, overlap little.
+// Which batches come here: pair_pays in d3q19.cu.
 #pragma once
 
 #include "pair_ops.cuh"

@@ -16,8 +16,8 @@
 // Every cell's arithmetic is that of step_kernel, operation by operation, and FP16 storage is rounded to
 // FP16 after every step, so a fused pass gives the same bits as single steps.
 //
-// What bounds it, on 4096 x 4096: FP32 moves 76 bytes per cell and pass plus 7 % of repeated halo rows
-// and runs at 6.3 TB/s (0.93 of the measured copy rate); the packed multiply-adds, two clocks each, keep
+// What bounds it, on 4096 x 4096: FP32 moves 1275 MB a pass (76 bytes per cell, 6 % of the reads repeated halo
+// rows) at 6.0 TB/s, 0.88 of the measured copy rate; the packed multiply-adds, two clocks each, keep
 // the FMA pipe 60 % busy beside that. A pass of four steps takes 0.212 ms against 4 x 0.196 ms for single
 // steps. FP16 moves half as much but converts every value after every step and is bound by instruction
 // issue: 0.21 ms a pass against 4 x 0.117 ms. Rows reach shared memory through cp.async three positions
