@@ -278,11 +278,31 @@ static cudaError_t enqueue_tiles(lbm_grid *g, int n, int check_every, int *check
     return e;
 }
 
-// One launch of the tile kernel at a time on a device: its CTAs wait for one another, and nothing promises that those of
-// two such launches, on two streams and short of SMs, become resident in turn and not each in part. A call that
-// finds another thread's under way steps in passes, with the same bits.
+// The tile kernel's launches under way on a device together take no more CTAs than it has SMs, one each: the CTAs of a
+// launch wait for one another, and nothing promises that those of two launches, on two streams and short of SMs, become
+// resident in turn and not each in part. A call that finds no room steps in passes, with the same bits.
 constexpr int TILE_DEVICES = 64;
-static std::mutex g_tile_mu[TILE_DEVICES];
+static std::atomic<int> g_tile_ctas[TILE_DEVICES];
+struct TileTurn {
+    std::atomic<int> *taken = nullptr;
+    int ctas = 0;
+    bool take(const lbm_grid *g)
+    {
+        if (g->tiles.ntx == 0 || g->dev >= TILE_DEVICES) return false;
+        std::atomic<int> &n = g_tile_ctas[g->dev];
+        if (n.fetch_add(g->tiles.ctas) + g->tiles.ctas > g->sms) {
+            n.fetch_sub(g->tiles.ctas);
+            return false;
+        }
+        taken = &n;
+        ctas = g->tiles.ctas;
+        return true;
+    }
+    ~TileTurn()
+    {
+        if (taken) taken->fetch_sub(ctas);
+    }
+};
 
 // LBM_OK, unless the grid holds no valid state.
 static lbm_status valid_state(const lbm_grid *g)
@@ -688,14 +708,13 @@ lbm_status lbm_step(lbm_grid *g, int64_t max_steps, double tol_rel, int32_t chec
     bool converged = false, checked = false, as_bits = false;       // as_bits: how the last check left its result
     bool tiled = false;
     Outcome o{};
-    std::unique_lock<std::mutex> tile_turn;                         // until the launches are done
-    if (g->tiles.ntx > 0 && g->dev < TILE_DEVICES)
-        tile_turn = std::unique_lock<std::mutex>(g_tile_mu[g->dev], std::try_to_lock);
+    TileTurn turn;                                                  // until the launches are done
+    const bool room = turn.take(g);
     while (left > 0) {
         // one launch of the tile kernel runs up to the next value the host needs
         int64_t m = left < TILE_CHUNK ? left : TILE_CHUNK;
         if (tol_rel > 0.0) m = std::min<int64_t>(m, check_every - g->t % check_every);
-        if (tile_turn.owns_lock() && g->tiles.ntx > 0 && m >= tiles_from(g->tiles)) {
+        if (room && g->tiles.ntx > 0 && m >= tiles_from(g->tiles)) {
             int checks = 0;
             const cudaError_t e = enqueue_tiles(g, (int)m, check_every, &checks);
             if (e == cudaErrorCooperativeLaunchTooLarge) {       // a stream with a part of the SMs

@@ -560,15 +560,16 @@ def test_runs_that_go_to_shared_memory(nx, ny, steps, resident):
         assert (lbm.lbm_launch_count() - n == 1) == resident
 
 
-def test_small_lattices_of_several_threads_at_once():
-    """Four threads step small lattices of their own on streams of their own. One of them at a time has its blocks wait
-    for one another in shared memory, the others go through passes; every state is that of the same run alone."""
+@pytest.mark.parametrize("nx,ny", [(400, 300), (40, 30)])
+def test_small_lattices_of_several_threads_at_once(nx, ny):
+    """Four threads step small lattices of their own on streams of their own: one that takes every SM, so that the others
+    go through passes meanwhile, and one of which several fit side by side. Every state is that of the same run alone."""
     import threading
 
     import torch
     lbm = _lbm()
-    kaps = [torch.from_numpy(synth.lognormal_kappa(400, 300, 4.0, 1.0, seed=40 + i).astype(np.float32)).cuda() for i in range(4)]
-    p = lbm.Params(nx=400, ny=300, tau=0.8, gx=1e-6)
+    kaps = [torch.from_numpy(synth.lognormal_kappa(nx, ny, 4.0, 1.0, seed=40 + i).astype(np.float32)).cuda() for i in range(4)]
+    p = lbm.Params(nx=nx, ny=ny, tau=0.8, gx=1e-6)
 
     def run(i, stream):
         with lbm.Grid(p, kaps[i], stream=stream) as G:
